@@ -131,7 +131,10 @@ int dwf_reset_counters(dwf_ctx* ctx);
  * 2^4 hypercube tiles, two s-slices per thread with packed FP32 over the
  * pair (loads into registers, or staged in shared memory by cp.async with 2,
  * 4 or 8 neighbours in flight), CTAs of 2 or 4 y-rows, the scalar form
- * with an L2 prefetch of the rows a CTA a wave later reads first; DWF_HOP_VARIANTS
+ * with an L2 prefetch of the rows a CTA a wave later reads first; id 0 is the
+ * untuned choice by lattice size: a kernel that streams the lattice along t
+ * through shared memory where that fills the GPU, else the scalar form under
+ * 64 registers; DWF_HOP_VARIANTS
  * variants for FP32 and FP16
  * storage at Ls >= 16, one otherwise; for DWF_F64 the one FP64 kernel, or
  * with DWF_ARITH_FLOAT_FLOAT the float-float kernel under four register

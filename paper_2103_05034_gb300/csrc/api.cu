@@ -151,12 +151,13 @@ extern "C" int dwf_ctx_create(dwf_ctx** out, const int L[4], int Ls, double M5, 
   }
   if (rc == DWF_OK) {
     if (cudaMalloc(&c->dscal, S_NSCAL * sizeof(double)) != cudaSuccess ||
-        cudaMallocHost(&c->hscal, S_NSCAL * sizeof(double)) != cudaSuccess) {
+        cudaMallocHost(&c->hscal, (S_NSCAL + 1) * sizeof(double)) != cudaSuccess) {
       cudaGetLastError();
       rc = DWF_ENOMEM;
     }
   }
   if (rc == DWF_OK) rc = dwf_reserve_partials(c, 1 << 16);
+  if (rc == DWF_OK) c->hscal[S_NSCAL] = 0;
   cudaError_t e = cudaStreamSynchronize(st);
   if (tmp) cudaFree(tmp);
   if (rc == DWF_OK && e != cudaSuccess) rc = DWF_ECUDA;
@@ -196,11 +197,12 @@ int dwf_ctx_clone_ls(const dwf_ctx* src, int ls, dwf_ctx** out, cudaStream_t st)
       rc = DWF_ECUDA;
   }
   if (rc == DWF_OK && (cudaMalloc(&c->dscal, S_NSCAL * sizeof(double)) != cudaSuccess ||
-                       cudaMallocHost(&c->hscal, S_NSCAL * sizeof(double)) != cudaSuccess)) {
+                       cudaMallocHost(&c->hscal, (S_NSCAL + 1) * sizeof(double)) != cudaSuccess)) {
     cudaGetLastError();
     rc = DWF_ENOMEM;
   }
   if (rc == DWF_OK) rc = dwf_reserve_partials(c, 1 << 16);
+  if (rc == DWF_OK) c->hscal[S_NSCAL] = 0;
   if (rc == DWF_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = DWF_ECUDA;
   if (rc != DWF_OK) {
     dwf_ctx_destroy(c);
@@ -244,6 +246,15 @@ static void fill_fifth(const dwf_ctx* c, dwfk::HopParams& hp, const double* mf, 
   }
 }
 
+// DWF_ETIMEOUT once a bounded wait of an earlier hopping launch has given up
+// (the kernel raises the flag behind hscal; reported once).
+static int hop_wait_status(dwf_ctx* c) {
+  volatile int* f = (volatile int*)(c->hscal + S_NSCAL);
+  if (!*f) return DWF_OK;
+  *f = 0;
+  return dwf_fail(c, DWF_ETIMEOUT, "a bounded wait of the hopping kernel gave up");
+}
+
 int launch_hop(dwf_ctx* c, const HopLaunch& h, int prec, cudaStream_t st, int* nblocks) {
   if (h.nrhs < 1 || h.nrhs > DWF_MAX_RHS) return dwf_fail(c, DWF_EINVAL, "nrhs out of range");
   dwfk::HopParams hp;
@@ -285,11 +296,16 @@ int launch_hop(dwf_ctx* c, const HopLaunch& h, int prec, cudaStream_t st, int* n
   fill_fifth(c, hp, h.mf, h.nrhs);
   if (h.reduce) {
     const int SB = c->g.Ls >= 16 ? 8 : 128 / c->g.Ls;
-    const size_t nb = (size_t)((c->g.Vh + SB - 1) / SB) * h.nrhs;
+    // a partial per CTA, or per consumer warp of the streaming kernel
+    size_t nb = (size_t)((c->g.Vh + SB - 1) / SB);
+    if (nb < 4096) nb = 4096;
+    nb *= h.nrhs;
     int rc = dwf_reserve_partials(c, nb);
     if (rc) return rc;
   }
   hp.partials = c->partials;
+  hp.wait_err = (int*)(c->hscal + S_NSCAL);
+  if (int rc = hop_wait_status(c)) return rc;
   if (h.cheb_tp) {
     hp.cheb_mode = 1;
     hp.cheb_x = h.cheb_x;
@@ -681,7 +697,7 @@ int read_scalars(dwf_ctx* c, int first, int n, cudaStream_t st) {
   DWF_CUDA(c, cudaMemcpyAsync(c->hscal + first, c->dscal + first, n * sizeof(double),
                               cudaMemcpyDeviceToHost, st));
   DWF_CUDA(c, cudaStreamSynchronize(st));
-  return DWF_OK;
+  return hop_wait_status(c);
 }
 
 int norm2_dev(dwf_ctx* c, const void* a, int64_t n, int prec, int dst, cudaStream_t st) {

@@ -25,6 +25,9 @@
 //   Gamma_5    gamma_5 with s -> Ls-1-s on the store
 //   reduction  |out|^2 in FP64 per CTA
 #pragma once
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include "dwf_internal.cuh"
 
 namespace dwfk {
@@ -40,6 +43,7 @@ struct HopParams {
   int zc;  // traversal z-chunk (even divisor of L2; L2 = lexicographic order)
   int l2pf; // > 0: each CTA prefetches into L2 the input rows first read by the
             // CTA l2pf positions later in the traversal (scalar kernel only)
+  int* wait_err;  // host-mapped flag raised by a bounded wait that gave up (streaming kernel)
   int out_parity;
   float sg;  // +1: D_hop, -1: D_hop^dag
   double alpha;
@@ -306,7 +310,88 @@ __device__ __forceinline__ void minv_row_inplace(cpx<R>* row, bool fwd, R d, R m
   }
 }
 
-extern __shared__ __align__(16) unsigned char hop_dyn_smem[];
+// Store of the operator output v at (field offset base, slice s): the CG
+// update (v becomes the new residual), the Chebyshev step, Gamma_5 v or v.
+template <int P, int LS, class R>
+__device__ __forceinline__ void hop_store(cpx<R> (&v)[12], const HopParams& p, int rhs, size_t base, int s) {
+  typedef typename Prec<P>::S S;
+  if (p.cg_mode) {
+    // CG update on the operator output v = A p: x += alpha p, r -= alpha v
+    const size_t off = base + s;
+    S* xs = (S*)p.cg_x + off;
+    float2* xs32 = (float2*)p.cg_x + off;
+    S* rs = (S*)p.cg_r + off;
+    const S* ps = (const S*)p.cg_p + off;
+    const R alpha = (R)p.cg_alpha[(size_t)rhs * p.cg_astride];
+    const bool x32 = (P == DWF_F16S) && p.cg_x32;
+#pragma unroll
+    for (int c = 0; c < 12; c++) {
+      cpx<R> xv, rv = ld_c(rs + c * LS);
+      if (x32) {
+        const float2 t = xs32[c * LS];
+        xv = cmake<R>((R)t.x, (R)t.y);
+      } else {
+        xv = ld_c(xs + c * LS);
+      }
+      const cpx<R> pv = ld_c(ps + c * LS);
+      xv.re = fma(alpha, pv.re, xv.re);
+      xv.im = fma(alpha, pv.im, xv.im);
+      rv.re = fma(-alpha, v[c].re, rv.re);
+      rv.im = fma(-alpha, v[c].im, rv.im);
+      if (x32)
+        xs32[c * LS] = make_float2((float)xv.re, (float)xv.im);
+      else
+        st_c(xs + c * LS, xv);
+      st_c(rs + c * LS, rv);
+      v[c] = rv;
+    }
+    return;
+  }
+  const int so = p.g5r5 ? LS - 1 - s : s;
+  if (p.cheb_mode) {
+    const S* cx = (const S*)p.cheb_x + base;
+    S* ct = (S*)p.cheb_tp + base;
+    S* ca = p.cheb_acc ? (S*)p.cheb_acc + base : nullptr;
+    const R ta = (R)p.cheb_ta, tb = (R)p.cheb_tb, cc = (R)p.cheb_cacc;
+#pragma unroll
+    for (int c = 0; c < 12; c++) {
+      cpx<R> o = v[c];
+      if (p.g5r5 && c >= 6) {
+        o.re = -o.re;
+        o.im = -o.im;
+      }
+      const cpx<R> xv = ld_c(cx + c * LS + so), tv = ld_c(ct + c * LS + so);
+      cpx<R> w;
+      w.re = fma(ta, o.re, fma(tb, xv.re, -tv.re));
+      w.im = fma(ta, o.im, fma(tb, xv.im, -tv.im));
+      st_c(ct + c * LS + so, w);
+      if (ca) {
+        cpx<R> av = ld_c(ca + c * LS + so);
+        av.re = fma(cc, w.re, av.re);
+        av.im = fma(cc, w.im, av.im);
+        st_c(ca + c * LS + so, av);
+      }
+    }
+    return;
+  }
+  S* out = (S*)p.out + base;
+  if (p.g5r5) {
+#pragma unroll
+    for (int c = 0; c < 12; c++) {
+      cpx<R> o = v[c];
+      if (c >= 6) {
+        o.re = -o.re;
+        o.im = -o.im;
+      }
+      st_c(out + c * LS + so, o);
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 12; c++) st_c(out + c * LS + s, v[c]);
+  }
+}
+
+extern __shared__ __align__(128) unsigned char hop_dyn_smem[];
 
 // Bulk prefetch of [p, p + bytes) into L2 (p and bytes multiples of 16).
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
@@ -607,83 +692,7 @@ __global__ void __launch_bounds__(LS* SB* RY, (HopMinBlocks<LS, SB * RY, REGS>::
     }
   }
 
-  if (p.cg_mode) {
-    // CG update on the operator output v = A p: x += alpha p, r -= alpha v;
-    // v becomes the new residual for the reduction below
-    if (active) {
-      const size_t off = (size_t)rhs * p.rhs_stride + (size_t)site * 12 * LS + s;
-      S* xs = (S*)p.cg_x + off;
-      float2* xs32 = (float2*)p.cg_x + off;
-      S* rs = (S*)p.cg_r + off;
-      const S* ps = (const S*)p.cg_p + off;
-      const R alpha = (R)p.cg_alpha[(size_t)rhs * p.cg_astride];
-      const bool x32 = (P == DWF_F16S) && p.cg_x32;
-#pragma unroll
-      for (int c = 0; c < 12; c++) {
-        cpx<R> xv, rv = ld_c(rs + c * LS);
-        if (x32) {
-          const float2 t = xs32[c * LS];
-          xv = cmake<R>((R)t.x, (R)t.y);
-        } else {
-          xv = ld_c(xs + c * LS);
-        }
-        const cpx<R> pv = ld_c(ps + c * LS);
-        xv.re = fma(alpha, pv.re, xv.re);
-        xv.im = fma(alpha, pv.im, xv.im);
-        rv.re = fma(-alpha, v[c].re, rv.re);
-        rv.im = fma(-alpha, v[c].im, rv.im);
-        if (x32)
-          xs32[c * LS] = make_float2((float)xv.re, (float)xv.im);
-        else
-          st_c(xs + c * LS, xv);
-        st_c(rs + c * LS, rv);
-        v[c] = rv;
-      }
-    }
-  } else if (active && p.cheb_mode) {
-    const size_t base = (size_t)rhs * p.rhs_stride + (size_t)site * 12 * LS;
-    const int so = p.g5r5 ? LS - 1 - s : s;
-    const S* cx = (const S*)p.cheb_x + base;
-    S* ct = (S*)p.cheb_tp + base;
-    S* ca = p.cheb_acc ? (S*)p.cheb_acc + base : nullptr;
-    const R ta = (R)p.cheb_ta, tb = (R)p.cheb_tb, cc = (R)p.cheb_cacc;
-#pragma unroll
-    for (int c = 0; c < 12; c++) {
-      cpx<R> o = v[c];
-      if (p.g5r5 && c >= 6) {
-        o.re = -o.re;
-        o.im = -o.im;
-      }
-      const cpx<R> xv = ld_c(cx + c * LS + so), tv = ld_c(ct + c * LS + so);
-      cpx<R> w;
-      w.re = fma(ta, o.re, fma(tb, xv.re, -tv.re));
-      w.im = fma(ta, o.im, fma(tb, xv.im, -tv.im));
-      st_c(ct + c * LS + so, w);
-      if (ca) {
-        cpx<R> av = ld_c(ca + c * LS + so);
-        av.re = fma(cc, w.re, av.re);
-        av.im = fma(cc, w.im, av.im);
-        st_c(ca + c * LS + so, av);
-      }
-    }
-  } else if (active) {
-    S* out = (S*)p.out + (size_t)rhs * p.rhs_stride + (size_t)site * 12 * LS;
-    if (p.g5r5) {
-      const int so = LS - 1 - s;
-#pragma unroll
-      for (int c = 0; c < 12; c++) {
-        cpx<R> o = v[c];
-        if (c >= 6) {
-          o.re = -o.re;
-          o.im = -o.im;
-        }
-        st_c(out + c * LS + so, o);
-      }
-    } else {
-#pragma unroll
-      for (int c = 0; c < 12; c++) st_c(out + c * LS + s, v[c]);
-    }
-  }
+  if (active) hop_store<P, LS>(v, p, rhs, (size_t)rhs * p.rhs_stride + (size_t)site * 12 * LS, s);
 
   if (p.reduce) {
     PartialSum<R> ps;
@@ -781,6 +790,7 @@ __global__ void __launch_bounds__(128) mooee_kernel(typename Prec<P>::S* out,
 }  // namespace dwfk
 
 #include "dhop_pair.cuh"
+#include "dhop_stream.cuh"
 
 namespace dwfk {
 
@@ -790,8 +800,11 @@ struct HopShape {
 };
 
 // Tuning variants of the hopping kernel: (register cap, prefetch).  Variant 0
-// is the uncapped kernel; the autotuner (dwf_autotune) times the rest on the
-// context's lattice and keeps the fastest per precision.
+// is the untuned default: the streaming kernel by its rule (launch_hop_stream),
+// else the scalar kernel, in FP32 arithmetic with 64 registers (8 CTAs an SM;
+// uncapped it takes 143: one M_pc of 16^3x32x16 205 us against 163).  The
+// autotuner (dwf_autotune) times the rest on the context's lattice and keeps
+// the fastest per precision.
 static_assert(DWF_HOP_VARIANTS == 26, "variant table below");
 __host__ __device__ constexpr int hop_variant_regs(int v) {
   return v == 0 ? 0 : v == 1 ? 96 : v == 2 ? 80 : v == 3 ? 64 : v == 4 ? 128 : v == 5 ? 96 : v == 6 ? 64 : v == 7 ? 80
@@ -833,6 +846,7 @@ inline void hop_launch_smem(dim3 grid, int threads, size_t bytes, const HopParam
 template <int P, int LSV, int V>
 inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
   constexpr int SB = HopShape<LSV>::SB;
+  constexpr int REGS = V == 0 && (P == DWF_F32 || P == DWF_F16S) ? 64 : hop_variant_regs(V);
   constexpr int PF = hop_variant_pf(V);
   constexpr int RY = PF == 4 ? 1 : hop_variant_rows(V);
   constexpr size_t cb = sizeof(cpx<typename Prec<P>::R>);
@@ -841,10 +855,10 @@ inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
   const size_t bytes = ub > sb ? ub : sb;
   if constexpr (PF == 4 && hop_variant_depth(V) > 0) {
     constexpr int D = hop_variant_depth(V);
-    hop_launch_smem<hop_kernel_pair<P, LSV, SB, hop_variant_regs(V), D>>(
+    hop_launch_smem<hop_kernel_pair<P, LSV, SB, REGS, D>>(
         grid, LSV / 2 * SB, pair_smem_bytes<P, LSV, SB, D>(hp.inv_mode != 0), hp, st);
   } else if constexpr (PF == 4) {
-    hop_launch_smem<hop_kernel_pair<P, LSV, SB, hop_variant_regs(V)>>(grid, LSV / 2 * SB, bytes, hp, st);
+    hop_launch_smem<hop_kernel_pair<P, LSV, SB, REGS>>(grid, LSV / 2 * SB, bytes, hp, st);
   } else if constexpr (hop_variant_l2pf(V) > 0) {
     // prefetch distance: the given number of waves of resident CTAs
     static int resident = 0;  // CTAs per GPU, one per instantiation
@@ -852,16 +866,16 @@ inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
       int dev = 0, nsm = 0, per = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, hop_kernel<P, LSV, SB, hop_variant_regs(V), PF, RY>,
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, hop_kernel<P, LSV, SB, REGS, PF, RY>,
                                                     LSV * SB * RY, bytes);
       resident = nsm * (per > 0 ? per : 1);
       if (resident < 1) resident = 1;
     }
     HopParams h2 = hp;
     h2.l2pf = hop_variant_l2pf(V) * resident;
-    hop_launch_smem<hop_kernel<P, LSV, SB, hop_variant_regs(V), PF, RY>>(grid, LSV * SB * RY, bytes, h2, st);
+    hop_launch_smem<hop_kernel<P, LSV, SB, REGS, PF, RY>>(grid, LSV * SB * RY, bytes, h2, st);
   } else {
-    hop_launch_smem<hop_kernel<P, LSV, SB, hop_variant_regs(V), PF, RY>>(grid, LSV * SB * RY, bytes, hp, st);
+    hop_launch_smem<hop_kernel<P, LSV, SB, REGS, PF, RY>>(grid, LSV * SB * RY, bytes, hp, st);
   }
 }
 
@@ -912,8 +926,115 @@ inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream
   return DWF_OK;
 }
 
+// One tensor map: rank dimensions (elements, innermost first), byte strides of
+// the outer ones, box.  Elements of 4 or 8 bytes are copied as they are.
+inline bool stream_map(CUtensorMap* m, const void* base, int elem, int rank, const cuuint64_t* dim,
+                       const cuuint64_t* stride, const cuuint32_t* box) {
+  static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return (PFN_cuTensorMapEncodeTiled_v12000)f;
+  }();
+  if (!encode) return false;
+  const cuuint32_t one[5] = {1, 1, 1, 1, 1};
+  return encode(m, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_UINT32, rank, (void*)base, dim,
+                stride, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The streaming kernel (dhop_stream.cuh) where it is the faster one; false
+// where a register-resident kernel is to run.  What decides is the fill: the
+// share of the consumers' thread-steps that are spent on sites until the last
+// CTA ends (ragged segments, the last round of units, the runs' boundary
+// slices, two steps to start up).  One M_pc, streaming against the 64-register
+// kernel, us: FP32 24^3x48 Ls 8 357 / 556 (fill 0.96), Ls 24 1170 / 1357
+// (0.99), 16^3x32 Ls 16 147 / 163 (0.88), 12^3x24 Ls 16 69 / 64 (0.57): equal
+// near 0.63, 0.86 and 0.7 to 0.79.  FP16 storage halves the bytes but not the
+// arithmetic that bounds the kernel: 24^3x48 Ls 8 386 / 581, but 16^3x32 Ls 16
+// 153 / 149 and 24^3x48 Ls 24 1195 / 1147, so only Ls 8 streams.
+template <int P, int LS>
+constexpr double stream_min_fill() {
+  return LS == 8 ? 0.68 : LS == 16 ? 0.74 : 0.87;
+}
+
+template <int P, int LS>
+inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, int* nblocks) {
+  typedef StreamCfg<P, LS> C;
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    cudaFuncSetAttribute(hop_stream<P, LS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES);
+    return n;
+  }();
+  // fewer than three steps a CTA: not worth the count below
+  if (sms < 1 || (double)hp.Vh * nrhs < stream_min_fill<P, LS>() * sms * 5 * C::SITES) return false;
+  StreamGrid g;
+  g.nseg = (hp.Lxh + C::SX - 1) / C::SX;
+  g.ny = hp.L1 / 2;
+  g.nz = hp.L2 / 2;
+  const long long units = (long long)g.nseg * g.ny * g.nz * nrhs;
+  if (units * hp.L3 > 0x7fffffff) return false;
+  g.units = (int)units;
+  const int grid = g.units * hp.L3 < sms ? g.units * hp.L3 : sms;
+  g.rounds = g.units / grid;
+  g.head = hp.L3;
+  double steps = g.rounds * (hp.L3 + 0.8);
+  if (const int left = g.units % grid) {
+    // the head that ends soonest, a piece's two boundary slices counted as 0.8 of a step
+    double best = 1e300;
+    for (int h = 1; h <= hp.L3; h++) {
+      const double rest = (double)left * (hp.L3 - h) / (grid - left);
+      const double share = h < hp.L3 ? rest + 0.8 * (1 + rest / (hp.L3 - h)) : 0.0;
+      const double cost = share > h + 0.8 ? share : h + 0.8;
+      if (cost < best) {
+        best = cost;
+        g.head = h;
+      }
+    }
+    steps += best;
+  }
+  if ((double)hp.Vh * nrhs < stream_min_fill<P, LS>() * sms * (steps + 2) * C::SITES) return false;
+  g.err = hp.wait_err;
+  double q = 1.0;
+  for (int k = 0; k < 25; k++, q /= hp.d) g.dp[k] = (float)q;
+  StreamMaps m;
+  {
+    const cuuint64_t row = (cuuint64_t)hp.Lxh * 12 * LS * C::CB;
+    const cuuint64_t dim[5] = {LS, (cuuint64_t)12 * hp.Lxh, (cuuint64_t)hp.L1, (cuuint64_t)hp.L2 * hp.L3, (cuuint64_t)nrhs};
+    const cuuint64_t str[4] = {LS * C::CB, row, row * hp.L1, (cuuint64_t)hp.rhs_stride * C::CB};
+    constexpr cuuint32_t RE = C::RB / C::CB;
+    const cuuint32_t bc[5] = {RE, 12 * C::SX, 2, 2, 1}, bs[5] = {RE, 12, 1, 1, 1};
+    const cuuint32_t by[5] = {RE, 12 * C::SX, 1, 2, 1}, bz[5] = {RE, 12 * C::SX, 2, 1, 1};
+    const cuuint64_t lrow = (cuuint64_t)hp.Lxh * 576;
+    const cuuint64_t ldim[4] = {72, (cuuint64_t)hp.Lxh, (cuuint64_t)hp.L1, (cuuint64_t)hp.L2 * hp.L3};
+    const cuuint64_t lstr[3] = {576, lrow, lrow * hp.L1};
+    const cuuint32_t lbox[4] = {C::LSTR / 8, C::SX, 2, 2};
+    if (!stream_map(&m.centre, hp.in, C::CB, 5, dim, str, bc) || !stream_map(&m.site, hp.in, C::CB, 5, dim, str, bs) ||
+        !stream_map(&m.hy, hp.in, C::CB, 5, dim, str, by) || !stream_map(&m.hz, hp.in, C::CB, 5, dim, str, bz) ||
+        !stream_map(&m.links, hp.links, 8, 4, ldim, lstr, lbox))
+      return false;
+  }
+  if (nblocks) *nblocks = grid * C::NG * C::NWG * nrhs;
+  hop_stream<P, LS><<<grid, C::NT, C::BYTES, st>>>(hp, g, m);
+  return true;
+}
+
 template <int P>
 int launch_hop_prec(const HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nblocks) {
+  if constexpr (P == DWF_F32 || P == DWF_F16S) {
+    if (variant == 0) {
+      if (Ls == 8 && launch_hop_stream<P, 8>(hp, nrhs, st, nblocks)) return DWF_OK;
+      if constexpr (P == DWF_F32) {
+        if (Ls == 16 && launch_hop_stream<P, 16>(hp, nrhs, st, nblocks)) return DWF_OK;
+        if (Ls == 24 && launch_hop_stream<P, 24>(hp, nrhs, st, nblocks)) return DWF_OK;
+      }
+    }
+  }
   dim3 grid;
   grid.y = nrhs;
   grid.z = 1;
