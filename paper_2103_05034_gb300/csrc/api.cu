@@ -238,10 +238,13 @@ static int64_t half_elems(const dwf_ctx* c) { return c->g.Vh * 12 * c->g.Ls; }
 static void fill_fifth(const dwf_ctx* c, dwfk::HopParams& hp, const double* mf, int nrhs) {
   const double d = 5.0 - c->M5;
   hp.d = d;
+  hp.one_sweep = fabs(d) >= 1.0;
   for (int r = 0; r < nrhs && r < DWF_MAX_RHS; r++) {
     const double m = mf ? mf[r] : 0.0;
+    const double md = m * pow(d, -(double)c->g.Ls);
     hp.m[r] = m;
-    hp.kappa[r] = 1.0 / (1.0 + m * pow(d, -(double)c->g.Ls));
+    hp.kappa[r] = 1.0 / (1.0 + md);
+    if (!(fabs(md) <= 1.0)) hp.one_sweep = 0;
     hp.dls1[r] = pow(d, 1.0 - (double)c->g.Ls);
   }
 }
@@ -296,9 +299,11 @@ int launch_hop(dwf_ctx* c, const HopLaunch& h, int prec, cudaStream_t st, int* n
   fill_fifth(c, hp, h.mf, h.nrhs);
   if (h.reduce) {
     const int SB = c->g.Ls >= 16 ? 8 : 128 / c->g.Ls;
-    // a partial per CTA, or per consumer warp of the streaming kernel
+    // a partial per CTA, or per consumer warp of the streaming kernel (at most
+    // 16 on each of 152 SMs); FP64 launches of fewer than 16 * 152 CTAs run
+    // CTAs of an eighth of their sites
     size_t nb = (size_t)((c->g.Vh + SB - 1) / SB);
-    if (nb < 4096) nb = 4096;
+    if (nb < 8 * 16 * 152) nb = 8 * 16 * 152;
     nb *= h.nrhs;
     int rc = dwf_reserve_partials(c, nb);
     if (rc) return rc;

@@ -48,6 +48,7 @@ struct HopParams {
   float sg;  // +1: D_hop, -1: D_hop^dag
   double alpha;
   int aux_mode, inv_mode, g5r5, reduce;
+  int one_sweep;  // M_ee^-1 by one sweep (see minv_row_inplace)
   long long rhs_stride;
   double d;
   // fused CG update (cg_mode = 1): with v = the operator output A p,
@@ -282,11 +283,35 @@ __device__ __forceinline__ void minv_row(cpx<R>* row, bool fwd, R d, R m, R kapp
   }
 }
 
-// The same inverse in place with O(1) registers (shared-memory rows): a
-// forward pass leaves F_q in the row, the backward pass recovers
-// v_q = F_q - F_{q-1}/d, accumulates G and writes x_q = kappa/d (F_q - m G_q).
+// The same inverse in place with O(1) registers (shared-memory rows).
+// one_sweep: with G_q = (v_q + G_{q-1}) / d along the sweep, x_q = G_q -
+// m kappa d^-(q+1) G_last: one dependent pass and 7 operations per complex
+// number.  It is stable while |d| >= 1 and |m d^-Ls| <= 1 (the host checks);
+// elsewhere the two terms can cancel, and two opposed sweeps (12 operations)
+// are taken as in minv_row.
 template <class R, int LS>
-__device__ __forceinline__ void minv_row_inplace(cpx<R>* row, bool fwd, R d, R m, R kappa, R dls1) {
+__device__ __forceinline__ void minv_row_inplace(cpx<R>* row, bool fwd, R d, R m, R kappa, R dls1, bool one_sweep) {
+  if (one_sweep) {
+    const R dinv = R(1) / d;
+    cpx<R> g = cmake<R>(0, 0);
+#pragma unroll 4
+    for (int q = 0; q < LS; q++) {
+      cpx<R>& e = row[fwd ? q : LS - 1 - q];
+      g.re = fma(g.re, dinv, dinv * e.re);
+      g.im = fma(g.im, dinv, dinv * e.im);
+      e = g;
+    }
+    R w = -m * kappa;
+#pragma unroll 4
+    for (int q = 0; q < LS; q++) {
+      cpx<R>& e = row[fwd ? q : LS - 1 - q];
+      w *= dinv;
+      e = cmake<R>(fma(w, g.re, e.re), fma(w, g.im, e.im));
+    }
+    return;
+  }
+  // a forward pass leaves F_q in the row, the backward pass recovers
+  // v_q = F_q - F_{q-1}/d, accumulates G and writes x_q = kappa/d (F_q - m G_q)
   const R dinv = R(1) / d;
   const R kd = kappa * dinv;
   cpx<R> f = cmake<R>(0, 0);
@@ -682,7 +707,7 @@ __global__ void __launch_bounds__(LS* SB* RY, (HopMinBlocks<LS, SB * RY, REGS>::
       if ((TILE || RY > 1) || site0 + sl2 < p.Vh) {
         const bool fwd = (c2 < 6) != (p.inv_mode == 2);
         minv_row_inplace<R, LS>(stage + (sl2 * 12 + c2) * (LS + 1), fwd, (R)p.d, (R)p.m[rhs],
-                        (R)p.kappa[rhs], (R)p.dls1[rhs]);
+                        (R)p.kappa[rhs], (R)p.dls1[rhs], p.one_sweep);
       }
     }
     __syncthreads();
@@ -791,13 +816,26 @@ __global__ void __launch_bounds__(128) mooee_kernel(typename Prec<P>::S* out,
 
 #include "dhop_pair.cuh"
 #include "dhop_stream.cuh"
+#include "dhop_dirs.cuh"
 
 namespace dwfk {
 
 template <int LS>
 struct HopShape {
   static constexpr int SB = (LS >= 16) ? 8 : (128 / LS);
+  static constexpr int SB1 = LS == 24 ? 4 : 32 / LS;  // the smallest whole number of warps
 };
+
+// FP64 launches: an SM has so few FP64 units that a launch takes as long as its
+// fullest SM.  Up to HOP_F64_DIRS sites (4D sites x Ls x fields) the eight
+// directions go to different threads (hop_dirs_f64: M_pc of 4^4x8 26 us
+// against 79; equal near 10000, and 1.2 to 1.4 times slower where the units
+// are busy: 8^3x16x8 85 us a hop against 63).  Launches of fewer than
+// HOP_F64_SMALL CTAs of the default size run CTAs of SB1 sites, which spread
+// evenly: 8^3x16 Ls 8 72 -> 63 us a hop, Ls 24 218 -> 198.  With more rounds
+// the sizes are equal and the large CTAs read the links in longer runs.
+constexpr long long HOP_F64_DIRS = 8192;
+constexpr long long HOP_F64_SMALL = 16 * 152;
 
 // Tuning variants of the hopping kernel: (register cap, prefetch).  Variant 0
 // is the untuned default: the streaming kernel by its rule (launch_hop_stream),
@@ -807,7 +845,7 @@ struct HopShape {
 // the fastest per precision.
 static_assert(DWF_HOP_VARIANTS == 26, "variant table below");
 __host__ __device__ constexpr int hop_variant_regs(int v) {
-  return v == 0 ? 0 : v == 1 ? 96 : v == 2 ? 80 : v == 3 ? 64 : v == 4 ? 128 : v == 5 ? 96 : v == 6 ? 64 : v == 7 ? 80
+  return v <= 0 ? 0 : v == 1 ? 96 : v == 2 ? 80 : v == 3 ? 64 : v == 4 ? 128 : v == 5 ? 96 : v == 6 ? 64 : v == 7 ? 80
          : v == 8 ? 64 : v == 9 ? 80 : v == 10 ? 128 : v == 11 ? 112 : v == 12 ? 96 : v == 13 ? 0
          : v == 14 ? 64 : v == 15 ? 80 : v == 16 ? 64 : v == 17 ? 80 : v == 18 ? 56 : v == 19 ? 48
          : v == 23 ? 64 : v == 24 ? 64 : v == 25 ? 80 : 0;
@@ -843,9 +881,8 @@ inline void hop_launch_smem(dim3 grid, int threads, size_t bytes, const HopParam
   Kern<<<grid, threads, bytes, st>>>(hp);
 }
 
-template <int P, int LSV, int V>
+template <int P, int LSV, int V, int SB = HopShape<LSV>::SB>
 inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
-  constexpr int SB = HopShape<LSV>::SB;
   constexpr int REGS = V == 0 && (P == DWF_F32 || P == DWF_F16S) ? 64 : hop_variant_regs(V);
   constexpr int PF = hop_variant_pf(V);
   constexpr int RY = PF == 4 ? 1 : hop_variant_rows(V);
@@ -882,7 +919,19 @@ inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
 template <int P, int LSV>
 inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream_t st) {
   // FP64 is ALU-bound and the small-Ls cases are test sizes: one variant.
-  if constexpr (P == DWF_F64 || LSV < 16) {
+  if constexpr (P == DWF_F64) {
+    if (grid.x == (hp.Vh + HopShape<LSV>::SB1 - 1) / HopShape<LSV>::SB1)
+      launch_hop_v<P, LSV, 0, HopShape<LSV>::SB1>(hp, grid, st);
+    else
+      launch_hop_v<P, LSV, 0>(hp, grid, st);
+  } else if (variant == 0 && (P == DWF_F32 || P == DWF_F16S) &&
+             (long long)grid.x * grid.y <= 152LL * (65536 / (LSV * HopShape<LSV>::SB * 144))) {
+    // All CTAs resident at once without a register cap: more loads in flight a
+    // thread, and nothing waits for a slot.  One hop of a filter, uncapped
+    // against 64 registers: 6x10x4x16 Ls 8 7.9 / 9.9 us, 6x6x8x12 Ls 24 10.0 /
+    // 12.0; past one round 8^3x16 Ls 16 13.6 / 12.1, four fields 43.5 / 33.8.
+    launch_hop_v<P, LSV, -1>(hp, grid, st);
+  } else if constexpr (LSV < 16) {
     launch_hop_v<P, LSV, 0>(hp, grid, st);
   } else if constexpr (P == DWF_P_DF) {
     // float-float: the plain kernel with register caps 96 / 80 / 64 (more
@@ -973,6 +1022,7 @@ inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, in
   }();
   // fewer than three steps a CTA: not worth the count below
   if (sms < 1 || (double)hp.Vh * nrhs < stream_min_fill<P, LS>() * sms * 5 * C::SITES) return false;
+  if (hp.inv_mode && !hp.one_sweep) return false;
   StreamGrid g;
   g.nseg = (hp.Lxh + C::SX - 1) / C::SX;
   g.ny = hp.L1 / 2;
@@ -1044,6 +1094,16 @@ int launch_hop_prec(const HopParams& hp, int Ls, int nrhs, int variant, cudaStre
     const int ry = (P == DWF_F64 || P == DWF_P_DF || LSV < 16) ? 1 : hop_variant_rows(variant); \
     if (ry > 1 && (hp.Lxh % SB || hp.L1 % ry)) return DWF_EINVAL;                \
     grid.x = (hp.Vh + SB * ry - 1) / (SB * ry);                                  \
+    if constexpr (P == DWF_F64) {                                                \
+      if ((long long)hp.Vh * LSV * nrhs <= HOP_F64_DIRS) {                       \
+        grid.x = (hp.Vh + DirsCfg<LSV>::SITES - 1) / DirsCfg<LSV>::SITES;        \
+        if (nblocks) *nblocks = grid.x * grid.y;                                 \
+        hop_dirs_f64<LSV><<<grid, DirsCfg<LSV>::NT, 0, st>>>(hp);                \
+        return DWF_OK;                                                           \
+      }                                                                          \
+      if ((long long)grid.x * nrhs < HOP_F64_SMALL)                              \
+        grid.x = (hp.Vh + HopShape<LSV>::SB1 - 1) / HopShape<LSV>::SB1;          \
+    }                                                                            \
     if (nblocks) *nblocks = grid.x * grid.y;                                     \
     return launch_hop_ls<P, LSV>(hp, grid, variant, st);                         \
   }

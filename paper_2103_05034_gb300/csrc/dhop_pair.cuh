@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(LS / 2 * SB, (HopMinBlocks<LS / 2, SB, REGS>::
       if (site0 + sl2 < p.Vh) {
         const bool fwd = (c2 < 6) != (p.inv_mode == 2);
         minv_row_inplace<float, LS>(stage + (sl2 * 12 + c2) * (LS + 1), fwd, (float)p.d, (float)p.m[rhs],
-                                    (float)p.kappa[rhs], (float)p.dls1[rhs]);
+                                    (float)p.kappa[rhs], (float)p.dls1[rhs], p.one_sweep);
       }
     }
     __syncthreads();
