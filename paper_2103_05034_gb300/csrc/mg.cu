@@ -169,16 +169,37 @@ int chiral(dwf_ctx* c, void* out, const void* in, int sign, int prec, int nrhs, 
   return DWF_OK;
 }
 
+// CTAs that share a block's sites in the restriction and the prolongation: a
+// power of two up to 8 (a portable cluster), so that there are about 16 CTAs an
+// SM, with two sites a CTA at least.
+int block_split(const BlockGeom& g) {
+  int split = 1;
+  while (split < 8 && (long long)g.nc * split < 16 * 152 && g.b4 >= 4 * split) split *= 2;
+  return split;
+}
+
 // out[xc][j][k] = <X_j, Y_k>_block (face-restricted for d > 0), FP64 results.
 int block_inner(dwf_ctx* c, const BlockGeom& g, const void* X, int nx, const void* Y, int ny, int prec,
                 double2* out, long long out_bstride, int out_ld, int d, int accumulate, cudaStream_t st) {
   const long long fs = full_elems(c);
   c->launches++;
-  if (ny == 1 && d == 0 && !accumulate && nx <= 64 && (prec == DWF_F32 || prec == DWF_F64)) {
+  const bool vec16 = ((((uintptr_t)X | (uintptr_t)Y)) & 15) == 0;  // 16-byte loads of FP32 pairs
+  if (ny == 1 && d == 0 && !accumulate && nx <= 64 && ((prec == DWF_F32 && vec16) || prec == DWF_F64)) {
     // restriction of one field: nx dot products per block in one pass
-#define DWF_RESTRICT(PV, NXV)                                                                                  \
-  dwfmg::k_block_restrict<PV, NXV><<<g.nc, 256, 0, st>>>((const typename Prec<PV>::S*)X, fs, nx,               \
-                                                         (const typename Prec<PV>::S*)Y, out, out_bstride, out_ld, g)
+    const int split = block_split(g);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    cfg.gridDim = dim3((unsigned)(g.nc * split));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = split;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+#define DWF_RESTRICT(PV, NXV)                                                                              \
+  DWF_CUDA(c, cudaLaunchKernelEx(&cfg, dwfmg::k_block_restrict<PV, NXV>, (const typename Prec<PV>::S*)X, fs, nx, \
+                                 (const typename Prec<PV>::S*)Y, out, out_bstride, out_ld, g, split))
     if (prec == DWF_F32) {
       if (nx <= 8) DWF_RESTRICT(DWF_F32, 8);
       else if (nx <= 32) DWF_RESTRICT(DWF_F32, 32);
@@ -213,6 +234,17 @@ int block_combine(dwf_ctx* c, const BlockGeom& g, void* Y, int ny, int py, const
   if (nx * ny > 1024) return dwf_fail(c, DWF_EINVAL, "block combine too wide");
   const long long fs = full_elems(c);
   c->launches++;
+  const bool vec16 = ((((uintptr_t)X | (uintptr_t)Y)) & 15) == 0;
+  if (ny == 1 && px == py && ((px == DWF_F32 && vec16) || px == DWF_F64)) {
+    const int split = block_split(g);
+    if (px == DWF_F64)
+      dwfmg::k_block_prolong<DWF_F64><<<g.nc * split, 256, 0, st>>>((double2*)Y, (const double2*)X, fs, nx, M, m_bstride,
+                                                                    m_ld, g, accumulate, split);
+    else
+      dwfmg::k_block_prolong<DWF_F32><<<g.nc * split, 256, 0, st>>>((float2*)Y, (const float2*)X, fs, nx, M, m_bstride,
+                                                                    m_ld, g, accumulate, split);
+    return DWF_OK;
+  }
   if (px == DWF_F64 && py == DWF_F64)
     dwfmg::k_block_combine<DWF_F64, DWF_F64><<<g.nc, 256, 0, st>>>((double2*)Y, fs, ny, (const double2*)X, fs,
                                                                    nx, M, m_bstride, m_ld, g, accumulate);

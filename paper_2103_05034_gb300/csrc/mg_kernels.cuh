@@ -4,6 +4,8 @@
 // updates), the face-split hopping term used to build the 9-point little
 // Dirac operator, and the coarse stencil apply on CUDA cores.
 #pragma once
+#include <cooperative_groups.h>
+
 #include "dhop_impl.cuh"
 #include "dwf_internal.cuh"
 
@@ -154,22 +156,52 @@ __global__ void __launch_bounds__(256) k_block_inner(const typename Prec<P>::S* 
   }
 }
 
+// 16 bytes of a field: one complex number in FP64, two in FP32.
+template <int P>
+struct Vec16;
+template <>
+struct Vec16<DWF_F64> {
+  static constexpr int N = 1;
+  cpx<double> v[1];
+  __device__ __forceinline__ void ld(const double2* p) { v[0] = ld_c(p); }
+  __device__ __forceinline__ void st(double2* p) const { st_c(p, v[0]); }
+};
+template <>
+struct Vec16<DWF_F32> {
+  static constexpr int N = 2;
+  cpx<float> v[2];
+  __device__ __forceinline__ void ld(const float2* p) {
+    const float4 t = *(const float4*)p;
+    v[0] = cmake(t.x, t.y);
+    v[1] = cmake(t.z, t.w);
+  }
+  __device__ __forceinline__ void st(float2* p) const {
+    *(float4*)p = make_float4(v[0].re, v[0].im, v[1].re, v[1].im);
+  }
+};
+
 // Restriction of one field: out[xc][j] = sum over block xc of conj(X_j) Y,
 // for nx <= 64 basis fields (the Gram-matrix kernel above would compute 32
-// columns of which one is wanted).  One CTA per block, eight warps; warp w
-// owns the basis fields j = w*J .. w*J+J-1 (J = NX/8) and walks all of the
-// block's elements with its 32 lanes (coalesced), so every basis element is
-// read once; sums of 16 terms in the storage's arithmetic type are added in
-// FP64 and reduced across the warp in FP64.
+// columns of which one is wanted).  Bound by reading the basis once from HBM.
+// A cluster of CTAs shares a block's sites, eight warps a CTA; warp w owns the
+// basis fields j = w*J .. w*J+J-1 (J = NX/8) and its lanes read 16 bytes each
+// of a site's row.  Sums of at most 16 terms in the storage's arithmetic type
+// are added in FP64, reduced across the warp, and the cluster's first CTA adds
+// the others' totals from their shared memory in order.  32 fields of
+// 16^4x16, 4^4 blocks (3.2 GB): 640 us = 5.1 TB/s, against 2065 us with one CTA a
+// block, 8-byte loads and the site's offset worked out for every element.
 template <int P, int NX>
 __global__ void __launch_bounds__(256) k_block_restrict(const typename Prec<P>::S* X, long long xstride, int nx,
                                                         const typename Prec<P>::S* Y, double2* out,
-                                                        long long out_bstride, int out_ld, BlockGeom g) {
+                                                        long long out_bstride, int out_ld, BlockGeom g, int split) {
   typedef typename Prec<P>::R R;
+  typedef Vec16<P> V;
   constexpr int J = NX / 8;
-  const int xc = blockIdx.x;
+  __shared__ double2 tot[NX];
+  const int xc = blockIdx.x / split, part0 = blockIdx.x - xc * split;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int j0 = w * J;
+  const typename Prec<P>::S* Xw = X + (long long)j0 * xstride;
   double2 acc[J];
   cpx<R> part[J];
 #pragma unroll
@@ -177,31 +209,35 @@ __global__ void __launch_bounds__(256) k_block_restrict(const typename Prec<P>::
     acc[j] = make_double2(0, 0);
     part[j] = cmake<R>(0, 0);
   }
-  const int row_len = 12 * g.Ls;
-  const int nel = g.b4 * row_len;
-  int cnt = 0;
-  for (int e = lane; e < nel; e += 32) {
-    const int i = e / row_len, q = e - i * row_len;
+  const int nv = 12 * g.Ls / V::N;
+  int terms = 0;
+  for (int i = j0 < nx ? part0 : g.b4; i < g.b4; i += split) {  // (none for a warp without fields)
     bool face;
-    const long long off = block_site_offset(g, xc, i, 0, &face) + q;
-    const cpx<R> y = ld_c(Y + off);
+    const long long off = block_site_offset(g, xc, i, 0, &face);
+    for (int e = lane; e < nv; e += 32) {
+      V y, a[J];
+      y.ld(Y + off + e * V::N);
 #pragma unroll
-    for (int j = 0; j < J; j++) {
-      if (j0 + j < nx) {
-        const cpx<R> a = ld_c(X + (long long)(j0 + j) * xstride + off);
-        part[j].re = fma(a.re, y.re, part[j].re);
-        part[j].re = fma(a.im, y.im, part[j].re);
-        part[j].im = fma(a.re, y.im, part[j].im);
-        part[j].im = fma(-a.im, y.re, part[j].im);
-      }
-    }
-    if (++cnt == 16) {
-      cnt = 0;
+      for (int j = 0; j < J; j++) a[j].ld(Xw + (j0 + j < nx ? j : 0) * xstride + off + e * V::N);
 #pragma unroll
-      for (int j = 0; j < J; j++) {
-        acc[j].x += (double)part[j].re;
-        acc[j].y += (double)part[j].im;
-        part[j] = cmake<R>(0, 0);
+      for (int j = 0; j < J; j++)
+#pragma unroll
+        for (int k = 0; k < V::N; k++) {
+          const cpx<R> x = a[j].v[k], t = y.v[k];
+          part[j].re = fma(x.re, t.re, part[j].re);
+          part[j].re = fma(x.im, t.im, part[j].re);
+          part[j].im = fma(x.re, t.im, part[j].im);
+          part[j].im = fma(-x.im, t.re, part[j].im);
+        }
+      terms += V::N;
+      if (terms == 16) {
+        terms = 0;
+#pragma unroll
+        for (int j = 0; j < J; j++) {
+          acc[j].x += (double)part[j].re;
+          acc[j].y += (double)part[j].im;
+          part[j] = cmake<R>(0, 0);
+        }
       }
     }
   }
@@ -213,12 +249,82 @@ __global__ void __launch_bounds__(256) k_block_restrict(const typename Prec<P>::
       x += __shfl_down_sync(0xffffffffu, x, o);
       y += __shfl_down_sync(0xffffffffu, y, o);
     }
-    if (lane == 0 && j0 + j < nx) out[xc * out_bstride + (long long)(j0 + j) * out_ld] = make_double2(x, y);
+    if (lane == 0) tot[j0 + j] = make_double2(x, y);
+  }
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  const int t = threadIdx.x;
+  if (part0 == 0 && t < nx) {
+    double2 r = tot[t];
+    for (int q = 1; q < split; q++) {
+      const double2 o = *cl.map_shared_rank(&tot[t], q);
+      r.x += o.x;
+      r.y += o.y;
+    }
+    out[xc * out_bstride + (long long)t * out_ld] = r;
+  }
+  cl.sync();  // the totals stay until they are read
+}
+
+// Prolongation of one coarse vector: Y(site) (+)= sum_j X_j(site) M[xc][j],
+// j < nx <= 1024.  Bound by reading the basis once from HBM: each thread keeps
+// eight 16-byte loads in flight, the sites of a block are shared by `split`
+// CTAs.  32 fields of 16^4x16 (3.2 GB): 634 us = 5.1 TB/s, against 1062 us as the
+// general kernel below, which takes one CTA a block and 8-byte loads.
+template <int P>
+__global__ void __launch_bounds__(256) k_block_prolong(typename Prec<P>::S* Y, const typename Prec<P>::S* X,
+                                                       long long xstride, int nx, const double2* M,
+                                                       long long m_bstride, int m_ld, BlockGeom g, int accumulate,
+                                                       int split) {
+  typedef typename Prec<P>::R R;
+  typedef Vec16<P> V;
+  __shared__ cpx<R> sm[1024];
+  const int xc = blockIdx.x / split, part0 = blockIdx.x - xc * split;
+  for (int j = threadIdx.x; j < nx; j += 256) {
+    const double2 m = M[xc * m_bstride + (long long)j * m_ld];
+    sm[j] = cmake<R>((R)m.x, (R)m.y);
+  }
+  __syncthreads();
+  const int nv = 12 * g.Ls / V::N;
+  const int sites = (g.b4 - part0 + split - 1) / split;  // of this CTA
+  for (int e = threadIdx.x; e < sites * nv; e += 256) {
+    const int i = e / nv;
+    bool face;
+    const long long off = block_site_offset(g, xc, part0 + i * split, 0, &face) + (e - i * nv) * V::N;
+    cpx<R> r[V::N];
+#pragma unroll
+    for (int k = 0; k < V::N; k++) r[k] = cmake<R>(0, 0);
+#pragma unroll 8
+    for (int j = 0; j < nx; j++) {
+      V a;
+      a.ld(X + j * xstride + off);
+      const cpx<R> m = sm[j];
+#pragma unroll
+      for (int k = 0; k < V::N; k++) {
+        r[k].re = fma(a.v[k].re, m.re, r[k].re);
+        r[k].re = fma(-a.v[k].im, m.im, r[k].re);
+        r[k].im = fma(a.v[k].re, m.im, r[k].im);
+        r[k].im = fma(a.v[k].im, m.re, r[k].im);
+      }
+    }
+    V y;
+    if (accumulate) {
+      y.ld(Y + off);
+#pragma unroll
+      for (int k = 0; k < V::N; k++) {
+        r[k].re += y.v[k].re;
+        r[k].im += y.v[k].im;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < V::N; k++) y.v[k] = r[k];
+    y.st(Y + off);
   }
 }
 
 // Y_k(site) = sum_j X_j(site) M[xc][j][k] over every site of every block:
-// prolongation (M = coarse vector) and Cholesky-QR updates (M = R^-1).
+// prolongation of several vectors and Cholesky-QR updates (M = R^-1).
 // One CTA per block; M staged in shared memory (nx * ny <= 1024).
 // The arithmetic is FP64 when either side is stored in FP64 (the Gram-Schmidt
 // of the basis), FP32 otherwise (prolongation inside the V-cycle).
