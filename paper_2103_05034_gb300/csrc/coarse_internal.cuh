@@ -15,9 +15,8 @@ struct dwf_coarse {
   float* At4;    // tensor-core copy (complex-split form per quad of sites), built on first use
   float* Bt;     // tensor-core right-hand sides (real form, TF32), per apply
   size_t Bt_bytes;
-  int* err;      // device error flag of the tensor-core kernel (sticky)
-  int* err_host; // pinned mirror, copied after every tensor-core apply
-  cudaEvent_t err_ready;  // recorded after that copy
+  int* err;      // sticky error flag of the tensor-core kernel, host memory that it writes
+  cudaEvent_t err_ready;  // recorded after every tensor-core apply
   void* ws[6];
   size_t ws_bytes[6];
   int* cg_acc;   // when set: coarse CG runs without host synchronisation and

@@ -91,17 +91,22 @@ __global__ void k_tc_arrange(float* At, const float2* A, int nc) {
 // Pre-arranged right-hand sides: Bt[y][kg = 16][n = N][4] TF32, K index
 // k < 32 the real part and k >= 32 the imaginary part of in[y][k mod 32][n]
 // (the K-major no-swizzle layout of one site's 64 x N B block), so that the
-// main kernel fetches a neighbour's block with one bulk copy.
-__global__ void k_tc_arrange_in(float* Bt, const float2* in, int nc, int N) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (y, j, n)
-  if (e >= (long long)nc * TC_NB * N) return;
+// main kernel fetches a neighbour's block with one bulk copy; split: as
+// Bt[y][kg = 8][part][n][4], the two parts side by side in N.  A thread takes
+// four consecutive k of one column: 16-byte stores, consecutive threads on
+// consecutive columns.
+__global__ void k_tc_arrange_in(float4* Bt, const float2* in, int nc, int N, int split) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (y, kg, n), kg < 8
+  if (e >= (long long)nc * (TC_NB / 4) * N) return;
   const int n = (int)(e % N);
-  const int j = (int)((e / N) % TC_NB);
-  const long long y = e / ((long long)N * TC_NB);
-  const float2 v = in[e];
-  const int kre = j, kim = TC_NB + j;
-  Bt[((y * (TC_ROWS / 4) + kre / 4) * N + n) * 4 + (kre & 3)] = to_tf32(v.x);
-  Bt[((y * (TC_ROWS / 4) + kim / 4) * N + n) * 4 + (kim & 3)] = to_tf32(v.y);
+  const int kg = (int)((e / N) % (TC_NB / 4));
+  const long long y = e / ((long long)N * (TC_NB / 4));
+  const float2* src = in + (y * TC_NB + 4 * kg) * N + n;
+  const float2 a = src[0], b = src[N], c = src[2 * N], d = src[3 * N];
+  float4* dst = Bt + y * (TC_ROWS / 4) * N;
+  if (split) dst += kg * N;
+  dst[kg * N + n] = make_float4(to_tf32(a.x), to_tf32(b.x), to_tf32(c.x), to_tf32(d.x));
+  dst[(split ? kg + 1 : TC_NB / 4 + kg) * N + n] = make_float4(to_tf32(a.y), to_tf32(b.y), to_tf32(c.y), to_tf32(d.y));
 }
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -237,7 +242,7 @@ __global__ void __launch_bounds__(TC_THREADS + 32, 1)
       for (int h = (nst > S - 1 ? nst - (S - 1) : 0); ok && h < nst; h++)
         if (!mma_stage(h)) ok = false;
       if (!ok) {
-        atomicExch(err, 1);
+        *(volatile int*)err = 1;
         atomicExch(&abort_flag, 1);
         // let copies still in flight land before the CTA exits (bounded)
         for (int h = (issued >= S ? issued - S : 0); h < issued; h++) mbar_wait(smem_u32(full + h % S), (h / S) & 1);
@@ -253,7 +258,7 @@ __global__ void __launch_bounds__(TC_THREADS + 32, 1)
       const int t = pl & 1;
       const int p = blockIdx.x + pl * gridDim.x;
       if (!mbar_wait(smem_u32(acc_full + t), (pl >> 1) & 1)) {
-        atomicExch(err, 1);
+        *(volatile int*)err = 1;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -284,17 +289,24 @@ __global__ void __launch_bounds__(TC_THREADS + 32, 1)
 
 // ---------------------------------------------------------------- complex-split form
 // The same stencil with the operator kept complex: per site and direction
-//   A' = [Re A | Im A]  (32 x 64),   B' = [[Re B, Im B], [-Im B, Re B]]  (64 x 2N),
-//   A' B' = [Re(A B) | Im(A B)],
-// so the operator streams at its complex FP32 size (half the real form's).
+//   A' = [Re A | Im A]  (32 x 64),   B = [Re B | Im B]  (32 x 2N),
+//   D1 = Re A B,  D2 = Im A B,   A B = D1_re - D2_im + i (D1_im + D2_re),
+// the last line in the epilogue, so that operator and right-hand sides stream
+// at their complex FP32 size.  With B as [[Re B, Im B], [-Im B, Re B]] (64 x
+// 2N) a stage was 96 KB instead of 64, and one thread issued copies and MMAs in
+// turn: 512 sites, 32 right-hand sides took 44.4 us a call.  The copies alone
+// take 20 us of a call, the MMAs alone 27 with 64 of N = 32 a stage (issue
+// bound), so the two are issued by different warps and the MMAs have N = 64:
+// 22.6 us.
 // One MMA tile (M = 128) stacks the A' of four consecutive coarse sites (a
-// quad); site q's neighbour block B'_q goes through the whole tile into
-// accumulator columns [q 2N, (q+1) 2N), whose rows 32q..32q+31 -- TMEM lanes
-// of epilogue warp q -- are site q's result.  One stage per (quad, direction):
+// quad); site q's neighbour block B_q goes through the whole tile into
+// accumulator columns [q 4N, (q+1) 4N) (D1, then D2), whose rows 32q..32q+31 --
+// TMEM lanes of epilogue warp q -- are site q's result.  One stage per (quad, direction):
 //   A: [K/4 = 16][M = 128][4] TF32, 32 KB, one bulk copy of the operator
 //      pre-arranged per quad;
-//   B: 4 x [K/4 = 16][2N][4] TF32 (N*512 B each), the neighbours' arranged blocks.
-// Accumulator: 4 x 2N columns, double buffered (N <= 32).
+//   B: 4 x [K/4 = 8][2N][4] TF32 (N*256 B each), the neighbours' arranged blocks.
+// Accumulator: 4 x 4N columns, double buffered for N = 16 (N = 32 takes all of
+// tensor memory).
 __global__ void k_tc4_arrange(float* At, const float2* A, int nc) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (x, d, j, k)
   if (e >= (long long)nc * 9 * TC_NB * TC_NB) return;
@@ -311,45 +323,30 @@ __global__ void k_tc4_arrange(float* At, const float2* A, int nc) {
   base[(((TC_NB + k) / 4) * TC_M + row) * 4 + ((TC_NB + k) & 3)] = to_tf32(a.y);  // K index 32 + k: Im A
 }
 
-__global__ void k_tc4_arrange_in(float* Bt, const float2* in, int nc, int N) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // (y, k, n)
-  if (e >= (long long)nc * TC_NB * N) return;
-  const int n = (int)(e % N);
-  const int k = (int)((e / N) % TC_NB);
-  const long long y = e / ((long long)N * TC_NB);
-  const float2 v = in[e];
-  const int N2 = 2 * N;
-  float* base = Bt + y * (TC_ROWS / 4) * N2 * 4;
-  auto put = [&](int kk, int nn, float val) { base[((kk / 4) * N2 + nn) * 4 + (kk & 3)] = to_tf32(val); };
-  put(k, n, v.x);
-  put(k, N + n, v.y);
-  put(TC_NB + k, n, -v.y);
-  put(TC_NB + k, N + n, v.x);
-}
-
 template <int N>
 struct Tc4Stages {
-  static constexpr int bytes = (TC_K / 4) * TC_M * 16 + 4 * (TC_K / 4) * (2 * N) * 16;
+  static constexpr int bytes = (TC_K / 4) * TC_M * 16 + 4 * (TC_K / 4) * N * 16;
   static constexpr int v = (220 * 1024 / bytes) < 4 ? (220 * 1024 / bytes) : 4;
 };
 
 // Persistent, warp-specialised as k_coarse_apply_tc, over quads instead of
-// pairs: warp 4 (one elected thread) issues each stage's five bulk copies and,
-// S-1 stages behind, its 32 MMAs (4 sites x 8 K-steps); warps 0-3 drain the
+// pairs: one thread of warp 4 issues each stage's five bulk copies, one of warp
+// 5 its 32 MMAs (4 sites x 4 K-steps x Re A, Im A); warps 0-3 drain the
 // accumulator, warp q writing site q of the quad.  Bounded waits as there.
 template <int N>
-__global__ void __launch_bounds__(TC_THREADS + 32, 1)
+__global__ void __launch_bounds__(TC_THREADS + 64, 1)
     k_coarse_apply_tc4(float2* out, const float* Bt, const float* At, int Lc0, int Lc1, int Lc2, int Lc3,
                        int nquads, int* err) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int S = Tc4Stages<N>::v;
   constexpr int N2 = 2 * N;
   constexpr int A_BYTES = (TC_K / 4) * TC_M * 16;  // 32 KB
-  constexpr int B_BYTES = (TC_K / 4) * N2 * 16;    // one site's B'
+  constexpr int B_BYTES = (TC_K / 4) * N * 16;     // one site's B
   constexpr int ST_BYTES = A_BYTES + 4 * B_BYTES;
   constexpr uint32_t LBO_A = TC_M * 16, LBO_B = N2 * 16, SBO = 128;
-  constexpr uint32_t NCOL = 4 * N2;  // one accumulator: four column ranges of 2N
-  constexpr uint32_t TCOLS = 2 * NCOL;
+  constexpr uint32_t NCOL = 4 * 2 * N2;  // one accumulator: four column ranges of 4N
+  constexpr int NBUF = NCOL <= 256 ? 2 : 1;
+  constexpr uint32_t TCOLS = NBUF * NCOL;
   static_assert(TCOLS <= 512 && (TCOLS & (TCOLS - 1)) == 0, "TMEM allocation is a power of two <= 512");
   static_assert(S >= 2, "at least two pipeline stages");
   uint64_t* bars = (uint64_t*)(smem + S * ST_BYTES);
@@ -380,39 +377,14 @@ __global__ void __launch_bounds__(TC_THREADS + 32, 1)
   constexpr uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N2 >> 3) << 17) |
                              ((uint32_t)(TC_M >> 4) << 24);
   const int myq = (int)blockIdx.x < nquads ? (nquads - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const int nst = myq * 9;
   if (warp == 4) {
     if (lane == 0) {
       bool ok = true;
-      const int nst = myq * 9;
       int issued = 0;
-      auto mma_stage = [&](int h) -> bool {
-        const int ql = h / 9, d = h % 9, t = ql & 1, b = h % S;
-        if (d == 0 && ql >= 2 && !mbar_wait(smem_u32(acc_empty + t), ((ql - 2) >> 1) & 1)) return false;
-        if (!mbar_wait(smem_u32(full + b), (h / S) & 1)) return false;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t a0 = smem_u32(smem + b * ST_BYTES);
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-          const uint32_t b0 = a0 + A_BYTES + q * B_BYTES;
-#pragma unroll
-          for (int kk = 0; kk < TC_K / 8; kk++) {
-            const uint64_t ad = smem_desc(a0 + kk * 2 * LBO_A, LBO_A, SBO);
-            const uint64_t bd = smem_desc(b0 + kk * 2 * LBO_B, LBO_B, SBO);
-            const uint32_t acc = (d > 0 || kk > 0) ? 1u : 0u;
-            asm volatile(
-                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + t * NCOL + q * N2),
-                "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                : "memory");
-          }
-        }
-        tc_commit(smem_u32(done + b));
-        if (d == 8) tc_commit(smem_u32(acc_full + t));
-        return true;
-      };
-      for (int g = 0; g < nst && ok; g++) {
-        const int ql = g / 9, d = g % 9, b = g % S;
-        const int qd = blockIdx.x + ql * gridDim.x;
+      for (int g = 0; g < nst; g++) {
+        const int d = g % 9, b = g % S;
+        const int qd = blockIdx.x + g / 9 * gridDim.x;
         if (g >= S && !mbar_wait(smem_u32(done + b), ((g - S) / S) & 1)) {
           ok = false;
           break;
@@ -423,47 +395,83 @@ __global__ void __launch_bounds__(TC_THREADS + 32, 1)
         bulk_g2s(smem_u32(st), At + ((long long)qd * 9 + d) * (TC_ROWS / 4) * TC_M * 4, A_BYTES, fb);
         for (int q = 0; q < 4; q++) {
           const int y = dwfmg::coarse_nbr(Lc, 4 * qd + q, d);
-          bulk_g2s(smem_u32(st + A_BYTES + q * B_BYTES), Bt + (long long)y * (TC_ROWS / 4) * N2 * 4, B_BYTES, fb);
+          bulk_g2s(smem_u32(st + A_BYTES + q * B_BYTES), Bt + (long long)y * (TC_ROWS / 4) * N * 4, B_BYTES, fb);
         }
         issued = g + 1;
-        if (g >= S - 1 && !mma_stage(g - (S - 1))) {
-          ok = false;
-          break;
-        }
       }
-      for (int h = (nst > S - 1 ? nst - (S - 1) : 0); ok && h < nst; h++)
-        if (!mma_stage(h)) ok = false;
       if (!ok) {
-        atomicExch(err, 1);
+        *(volatile int*)err = 1;
         atomicExch(&abort_flag, 1);
         for (int h = (issued >= S ? issued - S : 0); h < issued; h++) mbar_wait(smem_u32(full + h % S), (h / S) & 1);
       }
     }
+  } else if (warp == 5) {
+    if (lane == 0) {
+      for (int h = 0; h < nst; h++) {
+        const int ql = h / 9, d = h % 9, t = ql % NBUF, b = h % S;
+        if ((d == 0 && ql >= NBUF && !mbar_wait(smem_u32(acc_empty + t), ((ql - NBUF) / NBUF) & 1)) ||
+            !mbar_wait(smem_u32(full + b), (h / S) & 1)) {
+          *(volatile int*)err = 1;
+          atomicExch(&abort_flag, 1);
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t a0 = smem_u32(smem + b * ST_BYTES);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          const uint32_t b0 = a0 + A_BYTES + q * B_BYTES;
+#pragma unroll
+          for (int kk = 0; kk < TC_K / 8; kk++) {  // kk < 4: Re A into D1, else Im A into D2
+            const uint64_t ad = smem_desc(a0 + kk * 2 * LBO_A, LBO_A, SBO);
+            const uint64_t bd = smem_desc(b0 + (kk & 3) * 2 * LBO_B, LBO_B, SBO);
+            const uint32_t acc = (d > 0 || (kk & 3) > 0) ? 1u : 0u;
+            asm volatile(
+                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + t * NCOL + q * 2 * N2 +
+                                                                                     (kk >> 2) * N2),
+                "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                : "memory");
+          }
+        }
+        tc_commit(smem_u32(done + b));
+        if (d == 8) tc_commit(smem_u32(acc_full + t));
+      }
+    }
   } else {
     // epilogue: warp q owns TMEM lanes 32q..32q+31 = rows j of site 4 qd + q,
-    // columns [q 2N, q 2N + N) the real parts and [q 2N + N, (q+1) 2N) the imaginary
+    // columns q 4N + [0, N) Re A Re B, [N, 2N) Re A Im B, [2N, 3N) Im A Re B, [3N, 4N) Im A Im B
     const int q = warp, j = lane;
     for (int ql = 0; ql < myq; ql++) {
-      const int t = ql & 1;
+      const int t = ql % NBUF;
       const int qd = blockIdx.x + ql * gridDim.x;
-      if (!mbar_wait(smem_u32(acc_full + t), (ql >> 1) & 1)) {
-        atomicExch(err, 1);
+      if (!mbar_wait(smem_u32(acc_full + t), (ql / NBUF) & 1)) {
+        *(volatile int*)err = 1;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      float* o = (float*)(out + ((long long)(4 * qd + q) * TC_NB + j) * N);
+      float4* o = (float4*)(out + ((long long)(4 * qd + q) * TC_NB + j) * N);
 #pragma unroll
-      for (int c0 = 0; c0 < N2; c0 += 16) {
-        uint32_t v[16];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-            : "r"(tmem + t * NCOL + q * N2 + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
+      for (int c0 = 0; c0 < N; c0 += 16) {
+        uint32_t v[4][16];
+#pragma unroll
+        for (int part = 0; part < 4; part++) {
+          uint32_t* w = v[part];
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+              : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]),
+                "=r"(w[8]), "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15])
+              : "r"(tmem + t * NCOL + q * 2 * N2 + part * N + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
+        }
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const int part = c0 < N ? 0 : 1, n0 = c0 < N ? c0 : c0 - N;
 #pragma unroll
-        for (int i = 0; i < 16; i++) o[2 * (n0 + i) + part] = __uint_as_float(v[i]);
+        for (int i = 0; i < 16; i += 2) {
+          float4 r;
+          r.x = __uint_as_float(v[0][i]) - __uint_as_float(v[3][i]);
+          r.y = __uint_as_float(v[1][i]) + __uint_as_float(v[2][i]);
+          r.z = __uint_as_float(v[0][i + 1]) - __uint_as_float(v[3][i + 1]);
+          r.w = __uint_as_float(v[1][i + 1]) + __uint_as_float(v[2][i + 1]);
+          o[(c0 + i) / 2] = r;
+        }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(acc_empty + t)) : "memory");
@@ -507,7 +515,7 @@ int coarse_apply_tc(dwf_ctx* c, float2* out, const float2* in, const float2* A32
       k_tc4_arrange<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(*At4, A32, nc);
       c->launches++;
     }
-    const size_t bbytes = (size_t)nc * TC_ROWS * 2 * nrhs * sizeof(float);
+    const size_t bbytes = (size_t)nc * TC_ROWS * nrhs * sizeof(float);
     if (*Bt_bytes < bbytes) {
       if (*Bt) cudaFree(*Bt);
       *Bt = nullptr;
@@ -518,8 +526,8 @@ int coarse_apply_tc(dwf_ctx* c, float2* out, const float2* in, const float2* A32
       }
       *Bt_bytes = bbytes;
     }
-    const long long n = (long long)nc * TC_NB * nrhs;
-    k_tc4_arrange_in<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(*Bt, in, nc, nrhs);
+    const long long n = (long long)nc * (TC_NB / 4) * nrhs;
+    k_tc_arrange_in<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((float4*)*Bt, in, nc, nrhs, 1);
     c->launches += 2;
     const int nquads = nc / 4;
     const int grid = nquads < nsm ? nquads : nsm;
@@ -527,12 +535,12 @@ int coarse_apply_tc(dwf_ctx* c, float2* out, const float2* in, const float2* A32
     if (nrhs == 16) {
       smem = Tc4Stages<16>::v * Tc4Stages<16>::bytes + 256;
       cudaFuncSetAttribute(k_coarse_apply_tc4<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      k_coarse_apply_tc4<16><<<grid, TC_THREADS + 32, smem, st>>>(out, *Bt, *At4, Lc[0], Lc[1], Lc[2], Lc[3],
+      k_coarse_apply_tc4<16><<<grid, TC_THREADS + 64, smem, st>>>(out, *Bt, *At4, Lc[0], Lc[1], Lc[2], Lc[3],
                                                                    nquads, err_dev);
     } else {
       smem = Tc4Stages<32>::v * Tc4Stages<32>::bytes + 256;
       cudaFuncSetAttribute(k_coarse_apply_tc4<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      k_coarse_apply_tc4<32><<<grid, TC_THREADS + 32, smem, st>>>(out, *Bt, *At4, Lc[0], Lc[1], Lc[2], Lc[3],
+      k_coarse_apply_tc4<32><<<grid, TC_THREADS + 64, smem, st>>>(out, *Bt, *At4, Lc[0], Lc[1], Lc[2], Lc[3],
                                                                    nquads, err_dev);
     }
     return DWF_OK;
@@ -558,8 +566,8 @@ int coarse_apply_tc(dwf_ctx* c, float2* out, const float2* in, const float2* A32
     *Bt_bytes = bbytes;
   }
   {
-    const long long n = (long long)nc * TC_NB * nrhs;
-    k_tc_arrange_in<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(*Bt, in, nc, nrhs);
+    const long long n = (long long)nc * (TC_NB / 4) * nrhs;
+    k_tc_arrange_in<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((float4*)*Bt, in, nc, nrhs, 0);
     c->launches++;
   }
   const int npairs = nc / 2;

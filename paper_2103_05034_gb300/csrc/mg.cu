@@ -644,8 +644,7 @@ extern "C" int coarse_destroy(dwf_coarse* C) {
   if (C->Bt) cudaFree(C->Bt);
   if (C->Arb) cudaFree(C->Arb);
   coarse_defl_free(C);
-  if (C->err) cudaFree(C->err);
-  if (C->err_host) cudaFreeHost(C->err_host);
+  if (C->err) cudaFreeHost(C->err);
   if (C->err_ready) cudaEventDestroy(C->err_ready);
   for (int i = 0; i < 6; i++)
     if (C->ws[i]) cudaFree(C->ws[i]);
@@ -682,30 +681,26 @@ extern "C" int coarse_apply(dwf_coarse* C, void* out, const void* in, int nrhs, 
   if (prec != DWF_TF32) return dwf_fail(c, DWF_EINVAL, "coarse_apply precision: DWF_F32 or DWF_TF32");
   if (((uintptr_t)out & 15) || ((uintptr_t)in & 15)) return dwf_fail(c, DWF_EINVAL, "alignment");
   if (!C->err) {
-    if (cudaMalloc(&C->err, sizeof(int)) != cudaSuccess || cudaMallocHost(&C->err_host, sizeof(int)) != cudaSuccess ||
+    if (cudaMallocHost(&C->err, sizeof(int)) != cudaSuccess ||
         cudaEventCreateWithFlags(&C->err_ready, cudaEventDisableTiming) != cudaSuccess) {
       cudaGetLastError();
       return dwf_fail(c, DWF_ENOMEM, "coarse error flag");
     }
-    *C->err_host = 0;
-    DWF_CUDA(c, cudaMemsetAsync(C->err, 0, sizeof(int), st));
-    DWF_CUDA(c, cudaEventRecord(C->err_ready, st));
+    *C->err = 0;
   }
-  // The kernel's bounded waits report through a sticky device flag that is
-  // copied to pinned host memory after every apply; a flag raised by an
-  // earlier apply whose copy has landed is returned here, without waiting.
-  if (cudaEventQuery(C->err_ready) == cudaSuccess && *C->err_host) {
-    *C->err_host = 0;
-    DWF_CUDA(c, cudaMemsetAsync(C->err, 0, sizeof(int), st));
+  // The kernel's bounded waits report through a sticky flag in host memory
+  // that the kernel writes itself (a copy of a device flag after every apply
+  // cost 3 us a call); one raised by an earlier apply is returned here,
+  // without waiting.
+  if (*(volatile int*)C->err) {
+    *C->err = 0;
     return dwf_fail(c, DWF_ETIMEOUT, "tensor-core coarse apply: a bounded barrier wait gave up (earlier call)");
   }
-  cudaGetLastError();  // cudaEventQuery's cudaErrorNotReady is not an error
   int rc = coarse_apply_tc(c, (float2*)out, (const float2*)in, C->A32, &C->At, &C->At4, &C->Bt, &C->Bt_bytes, C->nb,
                            C->g.nc, C->g.Lc, nrhs, C->err, st);
   if (rc == DWF_EINVAL)
     return dwf_fail(c, rc, "tensor-core coarse apply needs nb = 32, an even number of coarse sites, nrhs 16/32/64");
   if (rc) return dwf_fail(c, rc, "tensor-core coarse apply");
-  DWF_CUDA(c, cudaMemcpyAsync(C->err_host, C->err, sizeof(int), cudaMemcpyDeviceToHost, st));
   DWF_CUDA(c, cudaEventRecord(C->err_ready, st));
   DWF_CUDA(c, cudaGetLastError());
   return DWF_OK;
@@ -715,12 +710,10 @@ extern "C" int coarse_apply_status(dwf_coarse* C, void* stream) {
   if (!C) return DWF_EINVAL;
   dwf_ctx* c = C->ctx;
   DWF_CUDA(c, cudaStreamSynchronize((cudaStream_t)stream));
-  if (!C->err_host) return DWF_OK;
+  if (!C->err) return DWF_OK;
   DWF_CUDA(c, cudaEventSynchronize(C->err_ready));
-  if (*C->err_host) {
-    *C->err_host = 0;
-    DWF_CUDA(c, cudaMemsetAsync(C->err, 0, sizeof(int), (cudaStream_t)stream));
-    DWF_CUDA(c, cudaStreamSynchronize((cudaStream_t)stream));
+  if (*(volatile int*)C->err) {
+    *C->err = 0;
     return dwf_fail(c, DWF_ETIMEOUT, "tensor-core coarse apply: a bounded barrier wait gave up");
   }
   return DWF_OK;
