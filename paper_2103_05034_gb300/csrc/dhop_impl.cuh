@@ -335,6 +335,28 @@ __device__ __forceinline__ void minv_row_inplace(cpx<R>* row, bool fwd, R d, R m
   }
 }
 
+// Store of the operator output v, or Gamma_5 v, at (field offset base, slice s).
+template <int P, int LS, class R>
+__device__ __forceinline__ void hop_put(const cpx<R> (&v)[12], const HopParams& p, size_t base, int s) {
+  typedef typename Prec<P>::S S;
+  const int so = LS - 1 - s;
+  S* out = (S*)p.out + base;
+  if (p.g5r5) {
+#pragma unroll
+    for (int c = 0; c < 12; c++) {
+      cpx<R> o = v[c];
+      if (c >= 6) {
+        o.re = -o.re;
+        o.im = -o.im;
+      }
+      st_c(out + c * LS + so, o);
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 12; c++) st_c(out + c * LS + s, v[c]);
+  }
+}
+
 // Store of the operator output v at (field offset base, slice s): the CG
 // update (v becomes the new residual), the Chebyshev step, Gamma_5 v or v.
 template <int P, int LS, class R>
@@ -399,21 +421,7 @@ __device__ __forceinline__ void hop_store(cpx<R> (&v)[12], const HopParams& p, i
     }
     return;
   }
-  S* out = (S*)p.out + base;
-  if (p.g5r5) {
-#pragma unroll
-    for (int c = 0; c < 12; c++) {
-      cpx<R> o = v[c];
-      if (c >= 6) {
-        o.re = -o.re;
-        o.im = -o.im;
-      }
-      st_c(out + c * LS + so, o);
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < 12; c++) st_c(out + c * LS + s, v[c]);
-  }
+  hop_put<P, LS>(v, p, base, s);
 }
 
 extern __shared__ __align__(128) unsigned char hop_dyn_smem[];
@@ -1000,45 +1008,40 @@ inline bool stream_map(CUtensorMap* m, const void* base, int elem, int rank, con
 // share of the consumers' thread-steps that are spent on sites until the last
 // CTA ends (ragged segments, the last round of units, the runs' boundary
 // slices, two steps to start up).  One M_pc, streaming against the 64-register
-// kernel, us: FP32 24^3x48 Ls 8 357 / 556 (fill 0.96), Ls 24 1170 / 1357
-// (0.99), 16^3x32 Ls 16 147 / 163 (0.88), 12^3x24 Ls 16 69 / 64 (0.57): equal
-// near 0.63, 0.86 and 0.7 to 0.79.  FP16 storage halves the bytes but not the
+// kernel, us: FP32 24^3x48 Ls 8 357 / 556 (fill 0.96), Ls 24 1055 / 1357
+// (0.99), 16^3x32 Ls 16 144 / 163 (0.88), 12^3x24 Ls 16 57 / 66 with rows of
+// three sites (0.77) but 69 / 64 with four (0.57), 12x16^3 Ls 16 72 / 72 (0.76):
+// equal near 0.63, 0.78 (Ls 24; the line stays where it was measured against
+// an earlier form, 1170 us) and 0.72.  FP16 storage halves the bytes but not the
 // arithmetic that bounds the kernel: 24^3x48 Ls 8 386 / 581, but 16^3x32 Ls 16
 // 153 / 149 and 24^3x48 Ls 24 1195 / 1147, so only Ls 8 streams.
+// The launches that end in a CG or Chebyshev step do not stream: their three
+// more fields are read by 12 to 16 warps an SM here against 32, and that costs
+// more than the hop gains: a filter of 16^3x32 Ls 16 123 us a hop if they
+// stream, 106 if not (109 with nothing streaming), a CG iteration 651, 628 and
+// 663 us.
 template <int P, int LS>
 constexpr double stream_min_fill() {
   return LS == 8 ? 0.68 : LS == 16 ? 0.74 : 0.87;
 }
 
-template <int P, int LS>
-inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, int* nblocks) {
-  typedef StreamCfg<P, LS> C;
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(hop_stream<P, LS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES);
-    return n;
-  }();
-  // fewer than three steps a CTA: not worth the count below
-  if (sms < 1 || (double)hp.Vh * nrhs < stream_min_fill<P, LS>() * sms * 5 * C::SITES) return false;
-  if (hp.inv_mode && !hp.one_sweep) return false;
-  StreamGrid g;
-  g.nseg = (hp.Lxh + C::SX - 1) / C::SX;
+// Decomposition for tiles of SX sites a row on sms CTAs; *fill as above.
+inline bool stream_grid(StreamGrid& g, const HopParams& hp, int nrhs, int SX, int sms, int* grid, double* fill) {
+  g.nseg = (hp.Lxh + SX - 1) / SX;
   g.ny = hp.L1 / 2;
   g.nz = hp.L2 / 2;
   const long long units = (long long)g.nseg * g.ny * g.nz * nrhs;
   if (units * hp.L3 > 0x7fffffff) return false;
   g.units = (int)units;
-  const int grid = g.units * hp.L3 < sms ? g.units * hp.L3 : sms;
-  g.rounds = g.units / grid;
+  *grid = g.units * hp.L3 < sms ? g.units * hp.L3 : sms;
+  g.rounds = g.units / *grid;
   g.head = hp.L3;
   double steps = g.rounds * (hp.L3 + 0.8);
-  if (const int left = g.units % grid) {
+  if (const int left = g.units % *grid) {
     // the head that ends soonest, a piece's two boundary slices counted as 0.8 of a step
     double best = 1e300;
     for (int h = 1; h <= hp.L3; h++) {
-      const double rest = (double)left * (hp.L3 - h) / (grid - left);
+      const double rest = (double)left * (hp.L3 - h) / (*grid - left);
       const double share = h < hp.L3 ? rest + 0.8 * (1 + rest / (hp.L3 - h)) : 0.0;
       const double cost = share > h + 0.8 ? share : h + 0.8;
       if (cost < best) {
@@ -1048,7 +1051,27 @@ inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, in
     }
     steps += best;
   }
-  if ((double)hp.Vh * nrhs < stream_min_fill<P, LS>() * sms * (steps + 2) * C::SITES) return false;
+  *fill = (double)hp.Vh * nrhs / (sms * (steps + 2) * 4 * SX);
+  return true;
+}
+
+template <int P, int LS, int SX>
+inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, int* nblocks) {
+  typedef StreamCfg<P, LS, SX> C;
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    cudaFuncSetAttribute(hop_stream<P, LS, SX>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES);
+    return n;
+  }();
+  // fewer than three steps a CTA: not worth the count below
+  if (sms < 1 || (double)hp.Vh * nrhs < stream_min_fill<P, LS>() * sms * 5 * C::SITES) return false;
+  if (hp.inv_mode && !hp.one_sweep) return false;
+  StreamGrid g;
+  int grid;
+  double fill;
+  if (!stream_grid(g, hp, nrhs, SX, sms, &grid, &fill) || fill < stream_min_fill<P, LS>()) return false;
   g.err = hp.wait_err;
   double q = 1.0;
   for (int k = 0; k < 25; k++, q /= hp.d) g.dp[k] = (float)q;
@@ -1070,18 +1093,19 @@ inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, in
       return false;
   }
   if (nblocks) *nblocks = grid * C::NG * C::NWG * nrhs;
-  hop_stream<P, LS><<<grid, C::NT, C::BYTES, st>>>(hp, g, m);
+  hop_stream<P, LS, SX><<<grid, C::NT, C::BYTES, st>>>(hp, g, m);
   return true;
 }
 
 template <int P>
 int launch_hop_prec(const HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nblocks) {
   if constexpr (P == DWF_F32 || P == DWF_F16S) {
-    if (variant == 0) {
-      if (Ls == 8 && launch_hop_stream<P, 8>(hp, nrhs, st, nblocks)) return DWF_OK;
+    if (variant == 0 && !hp.cheb_mode && !hp.cg_mode) {
+      if (Ls == 8 && launch_hop_stream<P, 8, 6>(hp, nrhs, st, nblocks)) return DWF_OK;
       if constexpr (P == DWF_F32) {
-        if (Ls == 16 && launch_hop_stream<P, 16>(hp, nrhs, st, nblocks)) return DWF_OK;
-        if (Ls == 24 && launch_hop_stream<P, 24>(hp, nrhs, st, nblocks)) return DWF_OK;
+        if (Ls == 16 && launch_hop_stream<P, 16, 4>(hp, nrhs, st, nblocks)) return DWF_OK;
+        if (Ls == 16 && launch_hop_stream<P, 16, 3>(hp, nrhs, st, nblocks)) return DWF_OK;
+        if (Ls == 24 && launch_hop_stream<P, 24, 2>(hp, nrhs, st, nblocks)) return DWF_OK;
       }
     }
   }

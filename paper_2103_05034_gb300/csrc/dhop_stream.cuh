@@ -1,5 +1,6 @@
 // Hopping term streamed along t through shared memory (arXiv:2103.05034,
-// Sec. 2, Eq. 2), with the epilogues of hop_kernel (same HopParams).
+// Sec. 2, Eq. 2), with the epilogues of hop_kernel (same HopParams) but the
+// CG and Chebyshev steps.
 //
 // One persistent CTA per SM walks units: a 2 x 2 (y, z) tile of x-segments of
 // up to SX checkerboard sites, all Ls slices, over a run of t.  Every input
@@ -30,9 +31,9 @@
 
 namespace dwfk {
 
-template <int P, int LS>
+template <int P, int LS, int SXV>
 struct StreamCfg {
-  static constexpr int SX = LS == 8 ? 6 : LS == 16 ? 4 : 2;       // sites per row of the tile
+  static constexpr int SX = SXV;                                  // sites per row of the tile
   static constexpr int SITES = 4 * SX;
   static constexpr int LPS = LS == 24 ? 8 : LS;                   // lanes per site and warp
   static constexpr int WPS = LS / LPS;                            // warps that share a site
@@ -275,10 +276,9 @@ __device__ __forceinline__ void stream_apply(f2p (&acc)[12], const f2p (&h)[6], 
 // holds spins 0,1 of both slices and the odd one spins 2,3: that halves the
 // shuffles of the scan.  The warps that share a site (Ls = 24) exchange their
 // totals through shared memory.
-template <int P, int LS>
+template <class C>
 __device__ __forceinline__ void stream_minv(cpx<float> (&v)[12], const HopParams& p, const StreamGrid& g, int rhs, int lq,
                                             int wq, int site, int grp, int buf) {
-  typedef StreamCfg<P, LS> C;
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int K = C::LPS / 2;                 // slice pairs of the warp's part
   const float dinv = g.dp[1];
@@ -351,11 +351,11 @@ __device__ __forceinline__ void stream_minv(cpx<float> (&v)[12], const HopParams
   }
 }
 
-template <int P, int LS>
-__global__ void __launch_bounds__(StreamCfg<P, LS>::NT, 1) hop_stream(const __grid_constant__ HopParams p,
+template <int P, int LS, int SXV>
+__global__ void __launch_bounds__(StreamCfg<P, LS, SXV>::NT, 1) hop_stream(const __grid_constant__ HopParams p,
                                                                     const __grid_constant__ StreamGrid g,
                                                                     const __grid_constant__ StreamMaps m) {
-  typedef StreamCfg<P, LS> C;
+  typedef StreamCfg<P, LS, SXV> C;
   typedef typename Prec<P>::S S;
   constexpr int SX = C::SX;
   const uint32_t bars = st_smem(C::OFF_B);
@@ -566,11 +566,6 @@ __global__ void __launch_bounds__(StreamCfg<P, LS>::NT, 1) hop_stream(const __gr
         const S* aux = (const S*)p.aux + base;
 #pragma unroll
         for (int c = 0; c < 12; c++) ax[c] = inside ? ld_c(aux + c * LS + s5) : cmake<float>(0.f, 0.f);
-        if (C::WPS > 1 && p.aux_mode > 1) {
-#pragma unroll
-          for (int c = 0; c < 12; c++)
-            ae[c] = inside ? ld_c(aux + c * LS + ((c < 6) != dagM ? sm : sp)) : cmake<float>(0.f, 0.f);
-        }
       }
       ok = ok && st_bar_wait(fullC((kc + 2) % 3), ((kc + 2) / 3) & 1);
       ld(c2 + offC);
@@ -601,6 +596,11 @@ __global__ void __launch_bounds__(StreamCfg<P, LS>::NT, 1) hop_stream(const __gr
             ae[c].re = __shfl_sync(0xffffffffu, ax[c].re, src);
             ae[c].im = __shfl_sync(0xffffffffu, ax[c].im, src);
           }
+        } else {  // (just read by other warps' lanes: L1 or L2)
+          const S* aux = (const S*)p.aux + base;
+#pragma unroll
+          for (int c = 0; c < 12; c++)
+            ae[c] = inside ? ld_c(aux + c * LS + ((c < 6) != dagM ? sm : sp)) : cmake<float>(0.f, 0.f);
         }
 #pragma unroll
         for (int c = 0; c < 12; c++) {
@@ -609,9 +609,9 @@ __global__ void __launch_bounds__(StreamCfg<P, LS>::NT, 1) hop_stream(const __gr
           v[c].im += fmaf(d, ax[c].im, co * ae[c].im);
         }
       }
-      if (p.inv_mode) stream_minv<P, LS>(v, p, g, w.rhs, lq, wq, st, grp, (kh >> 1) & 1);
+      if (p.inv_mode) stream_minv<C>(v, p, g, w.rhs, lq, wq, st, grp, (kh >> 1) & 1);
       if (inside && ok) {
-        hop_store<P, LS>(v, p, w.rhs, base, s5);
+        hop_put<P, LS>(v, p, base, s5);
         if (p.reduce) {
 #pragma unroll
           for (int c = 0; c < 12; c++) sum.add(fmaf(v[c].re, v[c].re, v[c].im * v[c].im));

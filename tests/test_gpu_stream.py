@@ -23,7 +23,7 @@ pytestmark = pytest.mark.gpu
 REF = 3
 SHAPES = [  # whole segments; ragged ones; a lattice of one y-tile
     ((24, 12, 8, 48), 8, F32), ((22, 12, 8, 64), 8, F32), ((24, 12, 8, 48), 8, F16S),
-    ((16, 16, 16, 16), 16, F32), ((14, 16, 16, 32), 16, F32), ((16, 2, 16, 192), 16, F32),
+    ((16, 16, 16, 16), 16, F32), ((14, 16, 16, 32), 16, F32), ((12, 12, 12, 24), 16, F32), ((16, 2, 16, 192), 16, F32),
     ((8, 16, 16, 48), 24, F32), ((34, 4, 8, 96), 24, F32),
 ]
 
