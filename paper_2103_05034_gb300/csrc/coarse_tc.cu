@@ -22,6 +22,7 @@
 
 #include "dwf_internal.cuh"
 #include "mg_kernels.cuh"
+#include "ring_roles.cuh"
 
 namespace {
 
@@ -144,8 +145,9 @@ struct TcStages {
 //     later, which reuses accumulator t (two accumulators of 2N columns in
 //     TMEM, so a pair's epilogue overlaps the next pair's MMAs).
 // Every wait is bounded; a thread whose wait runs out sets *err and stops
-// issuing work, and the producer waits (bounded) for copies still in flight
-// before the CTA frees its tensor memory.
+// issuing work, and the producer's last act is always to wait (bounded) for
+// its copies and MMAs, so that none is in flight when the CTA frees its tensor
+// memory, also where an epilogue warp gave up after the producer had issued all.
 template <int N>
 __global__ void __launch_bounds__(TC_THREADS + 32, 1)
     k_coarse_apply_tc(float2* out, const float* Bt, const float* At, int Lc0, int Lc1, int Lc2, int Lc3,
@@ -192,7 +194,7 @@ __global__ void __launch_bounds__(TC_THREADS + 32, 1)
     if (lane == 0) {
       bool ok = true;
       const int nst = mypairs * 9;
-      int issued = 0;  // stages whose copies were issued
+      int issued = 0, multiplied = 0;  // stages whose copies, whose MMAs were issued
       auto mma_stage = [&](int h) -> bool {
         const int pl = h / 9, d = h % 9, t = pl & 1, b = h % S;
         if (d == 0 && pl >= 2 && !mbar_wait(smem_u32(acc_empty + t), ((pl - 2) >> 1) & 1)) return false;
@@ -216,6 +218,7 @@ __global__ void __launch_bounds__(TC_THREADS + 32, 1)
         }
         tc_commit(smem_u32(done + b));
         if (d == 8) tc_commit(smem_u32(acc_full + t));
+        multiplied = h + 1;
         return true;
       };
       for (int g = 0; g < nst && ok; g++) {
@@ -244,9 +247,10 @@ __global__ void __launch_bounds__(TC_THREADS + 32, 1)
       if (!ok) {
         *(volatile int*)err = 1;
         atomicExch(&abort_flag, 1);
-        // let copies still in flight land before the CTA exits (bounded)
-        for (int h = (issued >= S ? issued - S : 0); h < issued; h++) mbar_wait(smem_u32(full + h % S), (h / S) & 1);
       }
+      // copies land and MMAs complete before the CTA exits, whoever gave up (bounded)
+      dwfk::ring_drain<S>((unsigned)issued, [&](int b, uint32_t par) { mbar_wait(smem_u32(full + b), par); });
+      if (multiplied > 0) mbar_wait(smem_u32(done + (multiplied - 1) % S), ((multiplied - 1) / S) & 1);
     }
   } else {
     // epilogue warps 0-3: warp w owns TMEM lanes 32w..32w+31 = stacked rows;
@@ -331,8 +335,10 @@ struct Tc4Stages {
 
 // Persistent, warp-specialised as k_coarse_apply_tc, over quads instead of
 // pairs: one thread of warp 4 issues each stage's five bulk copies, one of warp
-// 5 its 32 MMAs (4 sites x 4 K-steps x Re A, Im A); warps 0-3 drain the
-// accumulator, warp q writing site q of the quad.  Bounded waits as there.
+// 5 its 32 MMAs (4 sites x 4 K-steps x Re A, Im A), in the order of
+// ring_roles.cuh; warps 0-3 drain the accumulator, warp q writing site q of the
+// quad.  Bounded waits as there; each issuing warp waits at its end for what it
+// has issued, whoever gave up.
 template <int N>
 __global__ void __launch_bounds__(TC_THREADS + 64, 1)
     k_coarse_apply_tc4(float2* out, const float* Bt, const float* At, int Lc0, int Lc1, int Lc2, int Lc3,
@@ -378,64 +384,57 @@ __global__ void __launch_bounds__(TC_THREADS + 64, 1)
                              ((uint32_t)(TC_M >> 4) << 24);
   const int myq = (int)blockIdx.x < nquads ? (nquads - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int nst = myq * 9;
+  const auto wait_full = [&](int b, uint32_t par) { return mbar_wait(smem_u32(full + b), par); };
+  const auto wait_done = [&](int b, uint32_t par) { return mbar_wait(smem_u32(done + b), par); };
+  const auto raise = [&]() {
+    *(volatile int*)err = 1;
+    atomicExch(&abort_flag, 1);
+  };
   if (warp == 4) {
     if (lane == 0) {
-      bool ok = true;
-      int issued = 0;
-      for (int g = 0; g < nst; g++) {
-        const int d = g % 9, b = g % S;
-        const int qd = blockIdx.x + g / 9 * gridDim.x;
-        if (g >= S && !mbar_wait(smem_u32(done + b), ((g - S) / S) & 1)) {
-          ok = false;
-          break;
-        }
-        unsigned char* st = smem + b * ST_BYTES;
-        const uint32_t fb = smem_u32(full + b);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(ST_BYTES) : "memory");
-        bulk_g2s(smem_u32(st), At + ((long long)qd * 9 + d) * (TC_ROWS / 4) * TC_M * 4, A_BYTES, fb);
-        for (int q = 0; q < 4; q++) {
-          const int y = dwfmg::coarse_nbr(Lc, 4 * qd + q, d);
-          bulk_g2s(smem_u32(st + A_BYTES + q * B_BYTES), Bt + (long long)y * (TC_ROWS / 4) * N * 4, B_BYTES, fb);
-        }
-        issued = g + 1;
-      }
-      if (!ok) {
-        *(volatile int*)err = 1;
-        atomicExch(&abort_flag, 1);
-        for (int h = (issued >= S ? issued - S : 0); h < issued; h++) mbar_wait(smem_u32(full + h % S), (h / S) & 1);
-      }
+      dwfk::tc_copy_role<S>(
+          nst, wait_done, wait_full,
+          [&](int g, int b) {
+            const int d = g % 9;
+            const int qd = blockIdx.x + g / 9 * gridDim.x;
+            unsigned char* st = smem + b * ST_BYTES;
+            const uint32_t fb = smem_u32(full + b);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(ST_BYTES) : "memory");
+            bulk_g2s(smem_u32(st), At + ((long long)qd * 9 + d) * (TC_ROWS / 4) * TC_M * 4, A_BYTES, fb);
+            for (int q = 0; q < 4; q++) {
+              const int y = dwfmg::coarse_nbr(Lc, 4 * qd + q, d);
+              bulk_g2s(smem_u32(st + A_BYTES + q * B_BYTES), Bt + (long long)y * (TC_ROWS / 4) * N * 4, B_BYTES, fb);
+            }
+          },
+          raise);
     }
   } else if (warp == 5) {
     if (lane == 0) {
-      for (int h = 0; h < nst; h++) {
-        const int ql = h / 9, d = h % 9, t = ql % NBUF, b = h % S;
-        if ((d == 0 && ql >= NBUF && !mbar_wait(smem_u32(acc_empty + t), ((ql - NBUF) / NBUF) & 1)) ||
-            !mbar_wait(smem_u32(full + b), (h / S) & 1)) {
-          *(volatile int*)err = 1;
-          atomicExch(&abort_flag, 1);
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t a0 = smem_u32(smem + b * ST_BYTES);
+      dwfk::tc_mma_role<S, NBUF>(
+          nst, [&](int t, uint32_t par) { return mbar_wait(smem_u32(acc_empty + t), par); }, wait_full, wait_done,
+          [&](int h, int d, int t, int b) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t a0 = smem_u32(smem + b * ST_BYTES);
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-          const uint32_t b0 = a0 + A_BYTES + q * B_BYTES;
+            for (int q = 0; q < 4; q++) {
+              const uint32_t b0 = a0 + A_BYTES + q * B_BYTES;
 #pragma unroll
-          for (int kk = 0; kk < TC_K / 8; kk++) {  // kk < 4: Re A into D1, else Im A into D2
-            const uint64_t ad = smem_desc(a0 + kk * 2 * LBO_A, LBO_A, SBO);
-            const uint64_t bd = smem_desc(b0 + (kk & 3) * 2 * LBO_B, LBO_B, SBO);
-            const uint32_t acc = (d > 0 || (kk & 3) > 0) ? 1u : 0u;
-            asm volatile(
-                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + t * NCOL + q * 2 * N2 +
-                                                                                     (kk >> 2) * N2),
-                "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                : "memory");
-          }
-        }
-        tc_commit(smem_u32(done + b));
-        if (d == 8) tc_commit(smem_u32(acc_full + t));
-      }
+              for (int kk = 0; kk < TC_K / 8; kk++) {  // kk < 4: Re A into D1, else Im A into D2
+                const uint64_t ad = smem_desc(a0 + kk * 2 * LBO_A, LBO_A, SBO);
+                const uint64_t bd = smem_desc(b0 + (kk & 3) * 2 * LBO_B, LBO_B, SBO);
+                const uint32_t acc = (d > 0 || (kk & 3) > 0) ? 1u : 0u;
+                asm volatile(
+                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                    " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + t * NCOL + q * 2 * N2 +
+                                                                                         (kk >> 2) * N2),
+                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                    : "memory");
+              }
+            }
+            tc_commit(smem_u32(done + b));
+            if (d == 8) tc_commit(smem_u32(acc_full + t));
+          },
+          raise);
     }
   } else {
     // epilogue: warp q owns TMEM lanes 32q..32q+31 = rows j of site 4 qd + q,
