@@ -29,6 +29,8 @@
 
 #include <type_traits>
 
+#include "ring_roles.cuh"
+
 namespace dwfk {
 
 template <int P, int LS, int SXV>
@@ -390,75 +392,55 @@ __global__ void __launch_bounds__(StreamCfg<P, LS, SXV>::NT, 1) hop_stream(const
     if constexpr (C::REGSPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
     if (warp > C::NG * C::NWG) return;
     if (lane != 0) return;
-    unsigned kc = 0, kh = 0, kl = 0;
-    bool ok = true;
     StreamWork w(p, g);
-    while (ok && w.next(p, g)) {
-      const auto centre = [&](int i) {  // slice t0 - 1 + i
-        int t = w.t0 - 1 + i;
-        t = t < 0 ? t + L3 : t >= L3 ? t - L3 : t;
-        const int slot = kc % 3;
-        if (kc >= 3) ok = ok && st_bar_wait(emptyC(slot), (kc / 3 - 1) & 1);
-        if (!ok) return;
-        // the x-neighbours outside the segment are read in the slice's own step only
-        const bool ext = i > 0 && i <= w.nt && g.nseg > 1;
-        const uint32_t dst = st_smem(slot * C::CSLOT);
-        st_bar_expect(fullC(slot), C::COFF + (ext ? 4 * C::SS : 0));
-        st_copy5(dst, m.centre, 12 * w.xs, w.y0, t * L2 + w.z0, w.rhs, fullC(slot));
-        if (ext) {
-          const int left = w.xs == 0 ? Lxh - 1 : w.xs - 1, right = w.xs + w.len == Lxh ? 0 : w.xs + w.len;
-          const int b = (w.y0 + w.z0 + t + p.out_parity) & 1;  // of rows 0 and 3; rows 1 and 2 differ
+    const auto bar = [&](int ring, int slot, bool full) {
+      return ring == RING_C   ? (full ? fullC(slot) : emptyC(slot))
+             : ring == RING_L ? (full ? fullL(slot) : emptyL(slot))
+                              : (full ? fullH(slot, ring - RING_Y) : emptyH(slot, ring - RING_Y));
+    };
+    const auto centre = [&](int i, int slot) {  // slice t0 - 1 + i
+      int t = w.t0 - 1 + i;
+      t = t < 0 ? t + L3 : t >= L3 ? t - L3 : t;
+      // the x-neighbours outside the segment are read in the slice's own step only
+      const bool ext = i > 0 && i <= w.nt && g.nseg > 1;
+      const uint32_t dst = st_smem(slot * C::CSLOT);
+      st_bar_expect(fullC(slot), C::COFF + (ext ? 4 * C::SS : 0));
+      st_copy5(dst, m.centre, 12 * w.xs, w.y0, t * L2 + w.z0, w.rhs, fullC(slot));
+      if (ext) {
+        const int left = w.xs == 0 ? Lxh - 1 : w.xs - 1, right = w.xs + w.len == Lxh ? 0 : w.xs + w.len;
+        const int b = (w.y0 + w.z0 + t + p.out_parity) & 1;  // of rows 0 and 3; rows 1 and 2 differ
 #pragma unroll
-          for (int r = 0; r < 4; r++) {
-            const bool up = (b != 0) != (r == 1 || r == 2);
-            st_copy5(dst + C::COFF + r * C::SSA, m.site, 12 * (up ? right : left), w.y0 + (r & 1),
-                     t * L2 + w.z0 + (r >> 1), w.rhs, fullC(slot));
-          }
+        for (int r = 0; r < 4; r++) {
+          const bool up = (b != 0) != (r == 1 || r == 2);
+          st_copy5(dst + C::COFF + r * C::SSA, m.site, 12 * (up ? right : left), w.y0 + (r & 1), t * L2 + w.z0 + (r >> 1),
+                   w.rhs, fullC(slot));
         }
-        kc++;
-      };
-      const auto halo = [&](int i, int part) {
-        const int tz = (w.t0 + i) * L2;
-        const int slot = kh & 1;
-        if (kh >= 2) ok = ok && st_bar_wait(emptyH(slot, part), (kh / 2 - 1) & 1);
-        if (!ok) return;
-        const uint32_t dst = st_smem(C::OFF_H + slot * C::HSLOT), bar = fullH(slot, part);
-        constexpr int TWO = 2 * SX * C::SS;  // two rows
-        st_bar_expect(bar, 2 * TWO);
-        if (part == 0) {
-          st_copy5(dst, m.hy, 12 * w.xs, w.y0 == 0 ? L1 - 1 : w.y0 - 1, tz + w.z0, w.rhs, bar);
-          st_copy5(dst + TWO, m.hy, 12 * w.xs, w.y0 + 2 == L1 ? 0 : w.y0 + 2, tz + w.z0, w.rhs, bar);
-        } else {
-          st_copy5(dst + 2 * TWO, m.hz, 12 * w.xs, w.y0, tz + (w.z0 == 0 ? L2 - 1 : w.z0 - 1), w.rhs, bar);
-          st_copy5(dst + 3 * TWO, m.hz, 12 * w.xs, w.y0, tz + (w.z0 + 2 == L2 ? 0 : w.z0 + 2), w.rhs, bar);
-          kh++;
-        }
-      };
-      const auto links = [&](int i) {
-        const int slot = kl % 3;
-        if (kl >= 3) ok = ok && st_bar_wait(emptyL(slot), (kl / 3 - 1) & 1);
-        if (!ok) return;
-        st_bar_expect(fullL(slot), C::LSLOT);
-        st_copy4(st_smem(C::OFF_L + slot * C::LSLOT), m.links, w.xs, w.y0, (w.t0 + i) * L2 + w.z0, fullL(slot));
-        kl++;
-      };
-      centre(0);
-      centre(1);
-      for (int s = 0; ok && s < w.nt; s++) {
-        links(s);
-        if (ok) halo(s, 0);
-        if (ok) halo(s, 1);
-        if (ok) centre(s + 2);
       }
-    }
-    if (!ok) {  // a consumer did not free a slot: let the copies in flight land, then leave
-      *(volatile int*)g.err = 1;
-      for (unsigned k = kc > 3 ? kc - 3 : 0; k < kc; k++) st_bar_wait(fullC(k % 3), (k / 3) & 1);
-      for (unsigned k = kl > 3 ? kl - 3 : 0; k < kl; k++) st_bar_wait(fullL(k % 3), (k / 3) & 1);
-      for (unsigned k = kh > 2 ? kh - 2 : 0; k < kh; k++)
-        for (int h = 0; h < 2; h++) st_bar_wait(fullH(k & 1, h), (k / 2) & 1);
-      // (a y half without its z half is only left behind by a wait of the z half, which has outlasted the copy)
-    }
+    };
+    const auto halo = [&](int i, int part, int slot) {
+      const int tz = (w.t0 + i) * L2;
+      const uint32_t dst = st_smem(C::OFF_H + slot * C::HSLOT), bh = fullH(slot, part);
+      constexpr int TWO = 2 * SX * C::SS;  // two rows
+      st_bar_expect(bh, 2 * TWO);
+      if (part == 0) {
+        st_copy5(dst, m.hy, 12 * w.xs, w.y0 == 0 ? L1 - 1 : w.y0 - 1, tz + w.z0, w.rhs, bh);
+        st_copy5(dst + TWO, m.hy, 12 * w.xs, w.y0 + 2 == L1 ? 0 : w.y0 + 2, tz + w.z0, w.rhs, bh);
+      } else {
+        st_copy5(dst + 2 * TWO, m.hz, 12 * w.xs, w.y0, tz + (w.z0 == 0 ? L2 - 1 : w.z0 - 1), w.rhs, bh);
+        st_copy5(dst + 3 * TWO, m.hz, 12 * w.xs, w.y0, tz + (w.z0 + 2 == L2 ? 0 : w.z0 + 2), w.rhs, bh);
+      }
+    };
+    const auto links = [&](int i, int slot) {
+      st_bar_expect(fullL(slot), C::LSLOT);
+      st_copy4(st_smem(C::OFF_L + slot * C::LSLOT), m.links, w.xs, w.y0, (w.t0 + i) * L2 + w.z0, fullL(slot));
+    };
+    const auto wait_empty = [&](int ring, int slot, uint32_t par) { return st_bar_wait(bar(ring, slot, false), par); };
+    const auto wait_full = [&](int ring, int slot, uint32_t par) { return st_bar_wait(bar(ring, slot, true), par); };
+    const auto raise = [&]() { *(volatile int*)g.err = 1; };
+    // (order of the copies and their waits: ring_roles.cuh)
+    StreamProducer prod;
+    while (prod.ok && w.next(p, g)) prod.run(w.nt, wait_empty, centre, links, halo);
+    prod.finish(wait_full, raise);
     return;
   }
 

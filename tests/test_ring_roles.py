@@ -102,3 +102,71 @@ def _run(tmp_path, source):
 
 def test_coarse_stencil_roles_leave_nothing_in_flight(tmp_path):
     _run(tmp_path, TC)
+
+
+STREAM = r"""
+#include <cstdio>
+#include <set>
+#include <utility>
+#include <vector>
+#include "ring_roles.cuh"
+
+static int produce(const std::vector<int>& runs, int fail) {
+  const unsigned slots[4] = {3, 3, 2, 2};
+  unsigned issued[4] = {0, 0, 0, 0};
+  std::set<std::pair<int, unsigned>> landed;  // (ring, use)
+  int waits = 0, bad = 0;
+  bool gave_up = false, raised = false;
+  const auto issue = [&](int ring, int slot) {
+    if (gave_up || (unsigned)slot != issued[ring] % slots[ring]) bad++;
+    issued[ring]++;
+  };
+  dwfk::StreamProducer p;
+  for (int nt : runs) {
+    if (!p.ok) break;
+    p.run(
+        nt,
+        [&](int ring, int slot, unsigned par) {  // the use before the next one of the slot was read, so it had landed
+          const unsigned k = issued[ring] - slots[ring];
+          if ((unsigned)slot != k % slots[ring] || par != ((k / slots[ring]) & 1)) bad++;
+          if (waits++ >= fail) { gave_up = true; return false; }
+          landed.insert({ring, k});
+          return true;
+        },
+        [&](int, int slot) { issue(dwfk::RING_C, slot); }, [&](int, int slot) { issue(dwfk::RING_L, slot); },
+        [&](int, int part, int slot) { issue(dwfk::RING_Y + part, slot); });
+  }
+  p.finish(
+      [&](int ring, int slot, unsigned par) {
+        for (unsigned k = issued[ring]; k-- > 0;)
+          if (k % slots[ring] == (unsigned)slot) {
+            if (par == ((k / slots[ring]) & 1)) landed.insert({ring, k});
+            break;
+          }
+        return true;
+      },
+      [&]() { raised = true; });
+  for (int r = 0; r < 4; r++)
+    for (unsigned k = 0; k < issued[r]; k++)
+      if (!landed.count({r, k})) { std::printf("fail %d: ring %d use %u in flight\n", fail, r, k); bad++; }
+  return bad + (raised != gave_up);
+}
+
+int main() {
+  int bad = 0;
+  const std::vector<std::vector<int>> all = {{1}, {2}, {3}, {7}, {1, 1, 1}, {4, 2, 5}, {32, 5}};
+  for (const auto& runs : all) {
+    int n = 8;
+    for (int nt : runs) n += 4 * nt + 2;
+    for (int fail = 0; fail <= n; fail++) bad += produce(runs, fail);
+  }
+  std::printf("bad %d\n", bad);
+  return bad != 0;
+}
+"""
+
+
+def test_streaming_hop_producer_leaves_nothing_in_flight(tmp_path):
+    """Also where it is a consumer that gave up (no wait of the producer fails)
+    and where the z half of a halo step failed after its y half was issued."""
+    _run(tmp_path, STREAM)
