@@ -126,6 +126,19 @@ int64_t dwf_half_bytes(const dwf_ctx* ctx, int prec);
 int dwf_counters(const dwf_ctx* ctx, int64_t* launches, double* hop_bytes);
 int dwf_reset_counters(dwf_ctx* ctx);
 
+/* Hopping launches may wait inside the kernel (for copies into shared memory);
+ * every such wait is bounded.  One that gives up leaves the launch's output
+ * incomplete and raises a flag of the context, which is returned once as
+ * DWF_ETIMEOUT and then cleared: by dwf_status, by every call that
+ * synchronises (solvers, reductions, autotuner, setups, mg_smooth,
+ * mg_precondition), and by the next call that launches a hopping term.  The
+ * asynchronous entry points (dwf_dhop, dwf_mpc, dwf_mpcdag_mpc, dwf_ddw,
+ * dwf_hdw, cheby_filter, dwf_force, dwf_ratio_force) have returned DWF_OK by
+ * then, so a caller that synchronises by other means asks dwf_status whether
+ * what they wrote is whole.
+ * dwf_status synchronises `stream`. */
+int dwf_status(dwf_ctx* ctx, void* stream);
+
 /* Autotuner of the hopping kernel: times every tuning variant (register cap x
  * inner-loop form: scalar, neighbour prefetch, packed FP32 on (re, im) pairs,
  * 2^4 hypercube tiles, two s-slices per thread with packed FP32 over the
@@ -238,6 +251,10 @@ int dwf_norm2_noalloc(double* result, const void* a, int64_t n, int prec, void* 
  * expected outcome: the GPU stays usable and the status reaches the host),
  * DWF_OK if either wait unexpectedly completed.  Synchronises `stream`. */
 int dwf_selftest_wait_timeout(int* gave_up, void* stream);
+/* Self-test of the report of a hopping launch's wait that gave up (no
+ * counterpart in the paper): raises the context's flag from the host when
+ * `stream` reaches this call, as such a launch would from the device. */
+int dwf_selftest_raise_timeout(dwf_ctx* ctx, void* stream);
 
 /* Measured fused multiply-add rates of this GPU's CUDA cores (no counterpart
  * in the paper: the ALU roof for the FP64 hopping kernel and the FP64 parts
@@ -428,8 +445,9 @@ int coarse_export(const dwf_coarse* coarse, void* A, int* dims);
  * sites and nrhs in {16, 32, 64}; other shapes return DWF_EINVAL.  Both
  * paths are asynchronous on `stream`.  The tensor-core kernel's waits are
  * bounded: one that gives up raises a sticky flag of the operator, which a
- * later TF32 coarse_apply returns as DWF_ETIMEOUT once its copy to the host
- * has landed, and coarse_apply_status returns after synchronising. */
+ * later TF32 coarse_apply returns as DWF_ETIMEOUT without waiting (the kernel
+ * writes the flag to host memory), and coarse_apply_status after
+ * synchronising. */
 #define DWF_TF32 3
 int coarse_apply(dwf_coarse* coarse, void* out, const void* in, int nrhs, int prec, void* stream);
 /* Synchronise `stream` and return DWF_ETIMEOUT if a bounded wait of an

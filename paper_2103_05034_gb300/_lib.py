@@ -105,6 +105,7 @@ _SIGS = {
     "dwf_half_bytes": (I64, [P, I]),
     "dwf_counters": (I, [P, C.POINTER(I64), C.POINTER(D)]),
     "dwf_reset_counters": (I, [P]),
+    "dwf_status": (I, [P, P]),
     "dwf_autotune": (I, [P, I, I, C.POINTER(D), P]),
     "dwf_set_f64_arithmetic": (I, [P, I]),
     "dwf_get_f64_arithmetic": (I, [P]),
@@ -121,6 +122,7 @@ _SIGS = {
     "dwf_cdot": (I, [P, C.POINTER(D), P, P, I64, I, P]),
     "dwf_norm2_noalloc": (I, [C.POINTER(D), P, I64, I, P]),
     "dwf_selftest_wait_timeout": (I, [C.POINTER(C.c_int), P]),
+    "dwf_selftest_raise_timeout": (I, [P, P]),
     "dwf_measure_fma_peaks": (I, [C.POINTER(D), C.POINTER(D), P]),
     "rbcg_solve": (I, [P, P, P, D, D, I, I, C.POINTER(SolveStats), P]),
     "rbcg2_solve": (I, [P, P, P, D, D, I, I, C.POINTER(SolveStats), P]),

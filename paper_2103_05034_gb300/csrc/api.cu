@@ -157,7 +157,10 @@ extern "C" int dwf_ctx_create(dwf_ctx** out, const int L[4], int Ls, double M5, 
     }
   }
   if (rc == DWF_OK) rc = dwf_reserve_partials(c, 1 << 16);
-  if (rc == DWF_OK) c->hscal[S_NSCAL] = 0;
+  if (rc == DWF_OK) {
+    c->wait_flag = (int*)(c->hscal + S_NSCAL);
+    *c->wait_flag = 0;
+  }
   cudaError_t e = cudaStreamSynchronize(st);
   if (tmp) cudaFree(tmp);
   if (rc == DWF_OK && e != cudaSuccess) rc = DWF_ECUDA;
@@ -197,12 +200,12 @@ int dwf_ctx_clone_ls(const dwf_ctx* src, int ls, dwf_ctx** out, cudaStream_t st)
       rc = DWF_ECUDA;
   }
   if (rc == DWF_OK && (cudaMalloc(&c->dscal, S_NSCAL * sizeof(double)) != cudaSuccess ||
-                       cudaMallocHost(&c->hscal, (S_NSCAL + 1) * sizeof(double)) != cudaSuccess)) {
+                       cudaMallocHost(&c->hscal, S_NSCAL * sizeof(double)) != cudaSuccess)) {
     cudaGetLastError();
     rc = DWF_ENOMEM;
   }
   if (rc == DWF_OK) rc = dwf_reserve_partials(c, 1 << 16);
-  if (rc == DWF_OK) c->hscal[S_NSCAL] = 0;
+  c->wait_flag = src->wait_flag;  // (a clone lives within one call on its source)
   if (rc == DWF_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = DWF_ECUDA;
   if (rc != DWF_OK) {
     dwf_ctx_destroy(c);
@@ -249,13 +252,23 @@ static void fill_fifth(const dwf_ctx* c, dwfk::HopParams& hp, const double* mf, 
   }
 }
 
-// DWF_ETIMEOUT once a bounded wait of an earlier hopping launch has given up
-// (the kernel raises the flag behind hscal; reported once).
-static int hop_wait_status(dwf_ctx* c) {
-  volatile int* f = (volatile int*)(c->hscal + S_NSCAL);
+int dwf_wait_status(dwf_ctx* c) {
+  volatile int* f = c->wait_flag;
   if (!*f) return DWF_OK;
   *f = 0;
-  return dwf_fail(c, DWF_ETIMEOUT, "a bounded wait of the hopping kernel gave up");
+  return dwf_fail(c, DWF_ETIMEOUT, "a bounded wait of a hopping launch gave up: its output is incomplete");
+}
+
+extern "C" int dwf_status(dwf_ctx* c, void* stream) {
+  if (!c) return DWF_EINVAL;
+  DWF_CUDA(c, cudaStreamSynchronize((cudaStream_t)stream));
+  return dwf_wait_status(c);
+}
+
+extern "C" int dwf_selftest_raise_timeout(dwf_ctx* c, void* stream) {
+  if (!c) return DWF_EINVAL;
+  DWF_CUDA(c, cudaLaunchHostFunc((cudaStream_t)stream, [](void* f) { *(volatile int*)f = 1; }, c->wait_flag));
+  return DWF_OK;
 }
 
 int launch_hop(dwf_ctx* c, const HopLaunch& h, int prec, cudaStream_t st, int* nblocks) {
@@ -309,8 +322,8 @@ int launch_hop(dwf_ctx* c, const HopLaunch& h, int prec, cudaStream_t st, int* n
     if (rc) return rc;
   }
   hp.partials = c->partials;
-  hp.wait_err = (int*)(c->hscal + S_NSCAL);
-  if (int rc = hop_wait_status(c)) return rc;
+  hp.wait_err = c->wait_flag;
+  if (int rc = dwf_wait_status(c)) return rc;
   if (h.cheb_tp) {
     hp.cheb_mode = 1;
     hp.cheb_x = h.cheb_x;
@@ -463,7 +476,7 @@ extern "C" int dwf_autotune(dwf_ctx* c, int prec, int reps, double* best_ms, voi
   }
   if (best_ms) *best_ms = best_t;
   DWF_CUDA(c, cudaGetLastError());
-  return DWF_OK;
+  return dwf_wait_status(c);
 }
 
 extern "C" int dwf_counters(const dwf_ctx* c, int64_t* launches, double* hop_bytes) {
@@ -702,7 +715,7 @@ int read_scalars(dwf_ctx* c, int first, int n, cudaStream_t st) {
   DWF_CUDA(c, cudaMemcpyAsync(c->hscal + first, c->dscal + first, n * sizeof(double),
                               cudaMemcpyDeviceToHost, st));
   DWF_CUDA(c, cudaStreamSynchronize(st));
-  return hop_wait_status(c);
+  return dwf_wait_status(c);
 }
 
 int norm2_dev(dwf_ctx* c, const void* a, int64_t n, int prec, int dst, cudaStream_t st) {

@@ -128,6 +128,7 @@ struct dwf_ctx {
   size_t partials_n;
   double* dscal;      // device scalars for solvers
   double* hscal;      // pinned host mirror
+  int* wait_flag;     // behind hscal (a clone's: its source's): set by a kernel whose bounded wait gave up
   int hop_variant[3]; // tuned hopping-kernel variant per precision
   int f64_arith;      // FP64 hopping launches: DWF_ARITH_FP64 or DWF_ARITH_FLOAT_FLOAT
   double hop_l2_budget[3];  // L2 bytes the z-chunked traversal plans for (0: 48 MB)
@@ -252,6 +253,9 @@ int norm2_dev(dwf_ctx* c, const void* a, int64_t n, int prec, int dst, cudaStrea
 int mpc_apply(dwf_ctx* c, void* out, const void* in, void* tmp, const double* mf, int dagger, int prec,
               int nrhs, int reduce, cudaStream_t st, int* nparts);
 int read_scalars(dwf_ctx* c, int first, int n, cudaStream_t st);
+// DWF_ETIMEOUT, once, after a bounded wait of a hopping launch gave up, else
+// DWF_OK: after every synchronisation that hopping launches came before.
+int dwf_wait_status(dwf_ctx* c);
 // dscal[dst] = dscal[num] / dscal[den]
 int blas_scalar_div(dwf_ctx* c, int dst, int num, int den, cudaStream_t st);
 

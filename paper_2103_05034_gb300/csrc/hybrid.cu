@@ -941,6 +941,7 @@ int build_level1(dwf_hybrid* H, const void* eta4, cudaStream_t st) {
   if (rc == DWF_OK) {
     cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) rc = dwf_cuda_check(c, e, "4D filter");
+    if (rc == DWF_OK) rc = dwf_wait_status(c);  // (c4 shares the flag)
   }
   if (rc) {
     if (!c->err.size() && c4->err.size()) c->err = c4->err;

@@ -626,6 +626,7 @@ extern "C" int coarse_build(dwf_ctx* c, const void* basis, int nb, int nplus, co
   if (rc == DWF_OK) {
     cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) rc = dwf_cuda_check(c, e, "coarse_build");
+    if (rc == DWF_OK) rc = dwf_wait_status(c);
   }
   if (rc) {
     coarse_destroy(C);
@@ -941,6 +942,7 @@ int vgraph_build(VGraph& V, dwf_mg* G, cudaStream_t st) {
   V.acc_h[0] = V.acc_h[1] = 0;
   DWF_CUDA(c, cudaMemsetAsync(V.acc, 0, 2 * sizeof(int), st));
   DWF_CUDA(c, cudaStreamSynchronize(st));
+  if (int rc = dwf_wait_status(c)) return rc;  // of the warm-up V-cycle (the capture would take it for its own)
   const int64_t l0 = c->launches;
   double nH = 0;
   int nco = 0;
@@ -1068,6 +1070,7 @@ extern "C" int mg_setup(dwf_ctx* c, const dwf_mg_params* p, const void* eta, dwf
   if (rc == DWF_OK) {
     cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) rc = dwf_cuda_check(c, e, "mg_setup");
+    if (rc == DWF_OK) rc = dwf_wait_status(c);
   }
   G->setup_seconds = timer.sec();
   // 4. little Dirac operator of H_DW from the FP32 basis
@@ -1178,7 +1181,7 @@ extern "C" int mg_precondition(dwf_mg* G, void* out, const void* in, void* strea
   int rc = vcycle(G, out, in, (cudaStream_t)stream, &nH, &nc);
   if (rc) return rc;
   DWF_CUDA(G->ctx, cudaStreamSynchronize((cudaStream_t)stream));
-  return DWF_OK;
+  return dwf_wait_status(G->ctx);
 }
 
 extern "C" int mg_smooth(dwf_mg* G, void* out, const void* in, void* stream) {
@@ -1187,7 +1190,7 @@ extern "C" int mg_smooth(dwf_mg* G, void* out, const void* in, void* stream) {
   int rc = smoother(G, out, in, (cudaStream_t)stream, &nH);
   if (rc) return rc;
   DWF_CUDA(G->ctx, cudaStreamSynchronize((cudaStream_t)stream));
-  return DWF_OK;
+  return dwf_wait_status(G->ctx);
 }
 
 // Flexible GCR(nkrylov) on H_DW x = Gamma_5 b with the V(1,1) preconditioner;

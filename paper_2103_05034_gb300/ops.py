@@ -501,6 +501,12 @@ def dwf_measure_fma_peaks():
     return a.value, b.value
 
 
+def dwf_status(ctx):
+    """Synchronise and raise DWF_ETIMEOUT if a bounded wait of an earlier
+    hopping launch gave up (once)."""
+    check(lib().dwf_status(ctx.h, _stream()), ctx.h)
+
+
 def dwf_autotune(ctx, prec=F32, reps=20):
     """Pick the fastest hopping-kernel variant for this lattice; returns
     (variant, ms per launch)."""
