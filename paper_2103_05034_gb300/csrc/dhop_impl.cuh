@@ -29,6 +29,7 @@
 #include <cudaTypedefs.h>
 
 #include "dwf_internal.cuh"
+#include "per_device.cuh"
 
 namespace dwfk {
 
@@ -876,15 +877,34 @@ __host__ __device__ constexpr int hop_variant_pf(int v) {
   return v >= 23 ? 0 : v >= 20 ? 4 : v >= 14 ? 0 : v >= 10 ? 4 : v >= 8 ? 3 : v >= 6 ? 2 : v >= 4 ? 1 : 0;
 }  // 18, 19: scalar with 56 / 48 registers; 23-25: scalar with L2 prefetch
 
+// SMs of the current device (0: none).
+inline int device_sms() {
+  static PerDevice<int> cache;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const auto ask = [dev] {
+    int n = 0;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+  };
+  const int* n = cache.get(dev, ask);
+  return n ? *n : ask();
+}
+
 // Dynamic shared memory of one launch: links (SBC*72 complex, twice for the
 // (re,re,-im,im) packed form), or the M_ee^-1 stage (SBC*12*(LS+1) complex)
-// when the epilogue inverts; opted in above 48 KB once per instantiation.
+// when the epilogue inverts; above 48 KB every device is opted in, once per
+// instantiation, for the most that it can take.
 template <auto Kern>
-inline void hop_launch_smem(dim3 grid, int threads, size_t bytes, const HopParams& hp, cudaStream_t st) {
-  static size_t opted = 48 * 1024;  // one per kernel instantiation
-  if (bytes > opted) {
-    cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    opted = bytes;
+inline void hop_launch_smem(dim3 grid, int threads, size_t bytes, size_t most, const HopParams& hp, cudaStream_t st) {
+  if (most > 48 * 1024) {
+    static PerDevice<bool> opted;  // one per kernel instantiation
+    int dev = -1;
+    cudaGetDevice(&dev);
+    const auto opt_in = [most] {
+      return cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) == cudaSuccess;
+    };
+    if (!opted.get(dev, opt_in)) opt_in();
   }
   Kern<<<grid, threads, bytes, st>>>(hp);
 }
@@ -896,31 +916,31 @@ inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
   constexpr int RY = PF == 4 ? 1 : hop_variant_rows(V);
   constexpr size_t cb = sizeof(cpx<typename Prec<P>::R>);
   const size_t ub = (size_t)SB * RY * 72 * cb * (PF == 2 || PF == 4 ? 2 : 1);
-  const size_t sb = hp.inv_mode ? (size_t)SB * RY * 12 * (LSV + 1) * cb : 0;
-  const size_t bytes = ub > sb ? ub : sb;
+  const size_t sb = (size_t)SB * RY * 12 * (LSV + 1) * cb;
+  const size_t most = ub > sb ? ub : sb, bytes = hp.inv_mode ? most : ub;
   if constexpr (PF == 4 && hop_variant_depth(V) > 0) {
     constexpr int D = hop_variant_depth(V);
     hop_launch_smem<hop_kernel_pair<P, LSV, SB, REGS, D>>(
-        grid, LSV / 2 * SB, pair_smem_bytes<P, LSV, SB, D>(hp.inv_mode != 0), hp, st);
+        grid, LSV / 2 * SB, pair_smem_bytes<P, LSV, SB, D>(hp.inv_mode != 0), pair_smem_bytes<P, LSV, SB, D>(true), hp, st);
   } else if constexpr (PF == 4) {
-    hop_launch_smem<hop_kernel_pair<P, LSV, SB, REGS>>(grid, LSV / 2 * SB, bytes, hp, st);
+    hop_launch_smem<hop_kernel_pair<P, LSV, SB, REGS>>(grid, LSV / 2 * SB, bytes, most, hp, st);
   } else if constexpr (hop_variant_l2pf(V) > 0) {
     // prefetch distance: the given number of waves of resident CTAs
-    static int resident = 0;  // CTAs per GPU, one per instantiation
-    if (!resident) {
-      int dev = 0, nsm = 0, per = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, hop_kernel<P, LSV, SB, REGS, PF, RY>,
-                                                    LSV * SB * RY, bytes);
-      resident = nsm * (per > 0 ? per : 1);
-      if (resident < 1) resident = 1;
-    }
+    static PerDevice<int> cache;  // CTAs per GPU, one per instantiation
+    int dev = -1;
+    cudaGetDevice(&dev);
+    const auto count = [bytes] {
+      int per = 0;
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, hop_kernel<P, LSV, SB, REGS, PF, RY>, LSV * SB * RY, bytes);
+      const int n = device_sms() * (per > 0 ? per : 1);
+      return n > 0 ? n : 1;
+    };
+    const int* resident = cache.get(dev, count);
     HopParams h2 = hp;
-    h2.l2pf = hop_variant_l2pf(V) * resident;
-    hop_launch_smem<hop_kernel<P, LSV, SB, REGS, PF, RY>>(grid, LSV * SB * RY, bytes, h2, st);
+    h2.l2pf = hop_variant_l2pf(V) * (resident ? *resident : count());
+    hop_launch_smem<hop_kernel<P, LSV, SB, REGS, PF, RY>>(grid, LSV * SB * RY, bytes, most, h2, st);
   } else {
-    hop_launch_smem<hop_kernel<P, LSV, SB, REGS, PF, RY>>(grid, LSV * SB * RY, bytes, hp, st);
+    hop_launch_smem<hop_kernel<P, LSV, SB, REGS, PF, RY>>(grid, LSV * SB * RY, bytes, most, hp, st);
   }
 }
 
@@ -1058,13 +1078,17 @@ inline bool stream_grid(StreamGrid& g, const HopParams& hp, int nrhs, int SX, in
 template <int P, int LS, int SX>
 inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, int* nblocks) {
   typedef StreamCfg<P, LS, SX> C;
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(hop_stream<P, LS, SX>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES);
-    return n;
-  }();
+  static PerDevice<int> cache;  // SMs of a device that has opted in to the shared memory, else 0
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  const int* ready = cache.get(dev, [] {
+    if (cudaFuncSetAttribute(hop_stream<P, LS, SX>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return device_sms();
+  });
+  const int sms = ready ? *ready : 0;
   // fewer than three steps a CTA: not worth the count below
   if (sms < 1 || (double)hp.Vh * nrhs < stream_min_fill<P, LS>() * sms * 5 * C::SITES) return false;
   if (hp.inv_mode && !hp.one_sweep) return false;
@@ -1092,8 +1116,16 @@ inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, in
         !stream_map(&m.links, hp.links, 8, 4, ldim, lstr, lbox))
       return false;
   }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(C::NT);
+  cfg.dynamicSmemBytes = C::BYTES;
+  cfg.stream = st;
+  if (cudaLaunchKernelEx(&cfg, hop_stream<P, LS, SX>, hp, g, m) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
   if (nblocks) *nblocks = grid * C::NG * C::NWG * nrhs;
-  hop_stream<P, LS, SX><<<grid, C::NT, C::BYTES, st>>>(hp, g, m);
   return true;
 }
 
