@@ -125,6 +125,9 @@ int64_t dwf_half_bytes(const dwf_ctx* ctx, int prec);
  * complex spinor numbers + 72 link complex numbers).  Host-side, no sync. */
 int dwf_counters(const dwf_ctx* ctx, int64_t* launches, double* hop_bytes);
 int dwf_reset_counters(dwf_ctx* ctx);
+/* How many of the hopping-term launches since the last reset the streaming
+ * kernel took (the untuned choice decides by size; see dwf_autotune). */
+int dwf_streamed_launches(const dwf_ctx* ctx, int64_t* launches);
 
 /* Hopping launches may wait inside the kernel (for copies into shared memory);
  * every such wait is bounded.  One that gives up leaves the launch's output

@@ -105,6 +105,7 @@ _SIGS = {
     "dwf_half_bytes": (I64, [P, I]),
     "dwf_counters": (I, [P, C.POINTER(I64), C.POINTER(D)]),
     "dwf_reset_counters": (I, [P]),
+    "dwf_streamed_launches": (I, [P, C.POINTER(I64)]),
     "dwf_status": (I, [P, P]),
     "dwf_autotune": (I, [P, I, I, C.POINTER(D), P]),
     "dwf_set_f64_arithmetic": (I, [P, I]),

@@ -343,22 +343,24 @@ int launch_hop(dwf_ctx* c, const HopLaunch& h, int prec, cudaStream_t st, int* n
     hp.cg_x32 = h.cg_x32;
   }
   int rc;
+  bool streamed = false;
   switch (prec) {
     case DWF_F64:
       rc = c->f64_arith == DWF_ARITH_FLOAT_FLOAT ? dwf_launch_hop_df(hp, c->g.Ls, h.nrhs, c->hop_variant[0], st, nblocks)
                                                  : dwf_launch_hop_f64(hp, c->g.Ls, h.nrhs, c->hop_variant[0], st, nblocks);
       break;
     case DWF_F32:
-      rc = dwf_launch_hop_f32(hp, c->g.Ls, h.nrhs, c->hop_variant[1], st, nblocks);
+      rc = dwf_launch_hop_f32(hp, c->g.Ls, h.nrhs, c->hop_variant[1], st, nblocks, &streamed);
       break;
     case DWF_F16S:
-      rc = dwf_launch_hop_f16(hp, c->g.Ls, h.nrhs, c->hop_variant[2], st, nblocks);
+      rc = dwf_launch_hop_f16(hp, c->g.Ls, h.nrhs, c->hop_variant[2], st, nblocks, &streamed);
       break;
     default:
       return dwf_fail(c, DWF_EINVAL, "bad precision");
   }
   if (rc) return dwf_fail(c, rc, "unsupported Ls");
   c->launches++;
+  c->streamed += streamed;
   const double w = (double)dwf_complex_bytes(prec), wl = prec == DWF_F64 ? 16.0 : 8.0;
   c->hop_bytes += (double)c->g.Vh * ((double)c->g.Ls * h.nrhs * (24.0 + (h.aux_mode ? 12.0 : 0.0)) * w +
                                      72.0 * wl);
@@ -412,6 +414,7 @@ extern "C" int dwf_autotune(dwf_ctx* c, int prec, int reps, double* best_ms, voi
   float best_t = 1e30f;
   const int64_t launches0 = c->launches;
   const double bytes0 = c->hop_bytes;
+  const int64_t streamed0 = c->streamed;
   for (int v = 0; v < nv; v++) {
     if (!hop_variant_fits(c, prec, v)) continue;
     c->hop_variant[prec] = v;
@@ -467,6 +470,7 @@ extern "C" int dwf_autotune(dwf_ctx* c, int prec, int reps, double* best_ms, voi
   cudaEventDestroy(e1);
   c->launches = launches0;  // tuning launches are not counted
   c->hop_bytes = bytes0;
+  c->streamed = streamed0;
   // the two tuning fields are released (at 48^3 x 96 x 24 they are 24 GB)
   DWF_CUDA(c, cudaStreamSynchronize(st));
   for (int slot = 30; slot <= 31; slot++) {
@@ -486,10 +490,17 @@ extern "C" int dwf_counters(const dwf_ctx* c, int64_t* launches, double* hop_byt
   return DWF_OK;
 }
 
+extern "C" int dwf_streamed_launches(const dwf_ctx* c, int64_t* launches) {
+  if (!c || !launches) return DWF_EINVAL;
+  *launches = c->streamed;
+  return DWF_OK;
+}
+
 extern "C" int dwf_reset_counters(dwf_ctx* c) {
   if (!c) return DWF_EINVAL;
   c->launches = 0;
   c->hop_bytes = 0;
+  c->streamed = 0;
   return DWF_OK;
 }
 
@@ -825,7 +836,7 @@ struct CGGraph {
   cudaStream_t gs = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaGraphExec_t exec = nullptr;
-  int64_t launches = 0;
+  int64_t launches = 0, streamed = 0;
   double bytes = 0;
   int state = 0;  // 0: not built, 1: ready, -1: plain launches
   template <class F>
@@ -837,7 +848,7 @@ struct CGGraph {
       cudaGetLastError();
       return;
     }
-    const int64_t l0 = c->launches;
+    const int64_t l0 = c->launches, s0 = c->streamed;
     const double b0 = c->hop_bytes;
     const std::string err_before = c->err;
     cudaGraph_t g = nullptr;
@@ -849,8 +860,10 @@ struct CGGraph {
     for (int k = 0; k < n && rc == DWF_OK; k++) rc = body(gs);
     const cudaError_t ec = cudaStreamEndCapture(gs, &g);
     launches = c->launches - l0;
+    streamed = c->streamed - s0;
     bytes = c->hop_bytes - b0;
     c->launches = l0;
+    c->streamed = s0;
     c->hop_bytes = b0;
     if (rc || ec != cudaSuccess || !g || cudaGraphInstantiate(&exec, g, 0) != cudaSuccess) {
       if (g) cudaGraphDestroy(g);
@@ -869,6 +882,7 @@ struct CGGraph {
     DWF_CUDA(c, cudaEventRecord(e1, gs));
     DWF_CUDA(c, cudaStreamWaitEvent(st, e1, 0));
     c->launches += launches;
+    c->streamed += streamed;
     c->hop_bytes += bytes;
     return DWF_OK;
   }

@@ -1129,17 +1129,27 @@ inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, in
   return true;
 }
 
+// The streaming kernel, where a plain launch of this shape has one.
 template <int P>
-int launch_hop_prec(const HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nblocks) {
+bool try_hop_stream(const HopParams& hp, int Ls, int nrhs, cudaStream_t st, int* nblocks) {
   if constexpr (P == DWF_F32 || P == DWF_F16S) {
-    if (variant == 0 && !hp.cheb_mode && !hp.cg_mode) {
-      if (Ls == 8 && launch_hop_stream<P, 8, 6>(hp, nrhs, st, nblocks)) return DWF_OK;
-      if constexpr (P == DWF_F32) {
-        if (Ls == 16 && launch_hop_stream<P, 16, 4>(hp, nrhs, st, nblocks)) return DWF_OK;
-        if (Ls == 16 && launch_hop_stream<P, 16, 3>(hp, nrhs, st, nblocks)) return DWF_OK;
-        if (Ls == 24 && launch_hop_stream<P, 24, 2>(hp, nrhs, st, nblocks)) return DWF_OK;
-      }
+    if (hp.cheb_mode || hp.cg_mode) return false;
+    if (Ls == 8) return launch_hop_stream<P, 8, 6>(hp, nrhs, st, nblocks);
+    if constexpr (P == DWF_F32) {
+      if (Ls == 16)
+        return launch_hop_stream<P, 16, 4>(hp, nrhs, st, nblocks) || launch_hop_stream<P, 16, 3>(hp, nrhs, st, nblocks);
+      if (Ls == 24) return launch_hop_stream<P, 24, 2>(hp, nrhs, st, nblocks);
     }
+  }
+  return false;
+}
+
+template <int P>
+int launch_hop_prec(const HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nblocks,
+                    bool* streamed = nullptr) {
+  if (variant == 0 && try_hop_stream<P>(hp, Ls, nrhs, st, nblocks)) {
+    if (streamed) *streamed = true;
+    return DWF_OK;
   }
   dim3 grid;
   grid.y = nrhs;
@@ -1201,8 +1211,9 @@ int launch_mooee_prec(void* out, const void* in, const HopParams& hp, int dagger
 
 // Per-precision entry points (defined in dhop_f64.cu, dhop_f32.cu, dhop_f16.cu).
 int dwf_launch_hop_f64(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb);
-int dwf_launch_hop_f32(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb);
-int dwf_launch_hop_f16(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb);
+// (*streamed: the streaming kernel took the launch)
+int dwf_launch_hop_f32(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb, bool* streamed);
+int dwf_launch_hop_f16(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb, bool* streamed);
 // FP64 storage, float-float arithmetic (dhop_df.cu)
 int dwf_launch_hop_df(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb);
 int dwf_launch_mooee_f64(void* out, const void* in, const dwfk::HopParams& hp, int dagger,

@@ -134,6 +134,7 @@ struct dwf_ctx {
   double hop_l2_budget[3];  // L2 bytes the z-chunked traversal plans for (0: 48 MB)
   int64_t launches;   // kernel launches since the last counter reset
   double hop_bytes;   // algorithmic bytes of hopping-term launches
+  int64_t streamed;   // hopping launches that the streaming kernel took
   std::string err;
 };
 

@@ -908,7 +908,7 @@ struct VGraph {
   void* out = nullptr;
   int* acc = nullptr;    // device [coarse iterations, error bits]
   int* acc_h = nullptr;  // pinned mirror
-  int64_t launches = 0;  // kernel launches per replay
+  int64_t launches = 0, streamed = 0;  // kernel launches per replay, of them by the streaming kernel
   double nH = 0;         // H_DW applications per replay
   int state = 0;         // 0: not built, 1: ready, -1: not available
   int replays = 0;
@@ -943,7 +943,7 @@ int vgraph_build(VGraph& V, dwf_mg* G, cudaStream_t st) {
   DWF_CUDA(c, cudaMemsetAsync(V.acc, 0, 2 * sizeof(int), st));
   DWF_CUDA(c, cudaStreamSynchronize(st));
   if (int rc = dwf_wait_status(c)) return rc;  // of the warm-up V-cycle (the capture would take it for its own)
-  const int64_t l0 = c->launches;
+  const int64_t l0 = c->launches, s0 = c->streamed;
   double nH = 0;
   int nco = 0;
   cudaGraph_t graph = nullptr;
@@ -957,7 +957,9 @@ int vgraph_build(VGraph& V, dwf_mg* G, cudaStream_t st) {
   G->coarse->cg_acc = nullptr;
   const cudaError_t ec = cudaStreamEndCapture(V.gs, &graph);
   V.launches = c->launches - l0;
+  V.streamed = c->streamed - s0;
   c->launches = l0;
+  c->streamed = s0;
   if (rc || ec != cudaSuccess || !graph || cudaGraphInstantiate(&V.exec, graph, 0) != cudaSuccess) {
     // capture not possible (e.g. a launch form the CUDA driver cannot record):
     // the solve continues with plain launches
@@ -985,6 +987,7 @@ int vgraph_run(VGraph& V, void* z, const void* r, cudaStream_t st, double* nH) {
   DWF_CUDA(c, cudaMemcpyAsync(z, V.out, bytes, cudaMemcpyDeviceToDevice, st));
   DWF_CUDA(c, cudaMemcpyAsync(V.acc_h, V.acc, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   c->launches += V.launches;
+  c->streamed += V.streamed;
   *nH += V.nH;
   V.replays++;
   return DWF_OK;

@@ -88,6 +88,13 @@ def dwf_counters(ctx):
     return n.value, b.value
 
 
+def dwf_streamed_launches(ctx):
+    """Hopping launches that the streaming kernel took since the last reset."""
+    n = C.c_int64()
+    check(lib().dwf_streamed_launches(ctx.h, C.byref(n)))
+    return n.value
+
+
 def dwf_reset_counters(ctx):
     check(lib().dwf_reset_counters(ctx.h))
 
