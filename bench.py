@@ -110,9 +110,15 @@ def source_hash(*rel):
     return h.hexdigest()[:16]
 
 
+# The text of the hopping kernels: a traffic figure belongs to all of these files.
+HOP_KERNEL_SOURCES = tuple("paper_2103_05034_gb300/csrc/" + f for f in
+                           ("dhop_dirs.cuh", "dhop_impl.cuh", "dhop_pair.cuh", "dhop_stream.cuh", "ring_roles.cuh"))
+
+
 def profile_traffic(kernel_key, shash):
     """DRAM bytes per launch from the committed ncu summary, if it was taken on
-    the current kernel source."""
+    the current kernel source: shash, and the hash of every file of
+    HOP_KERNEL_SOURCES that the record carries."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
         return None
@@ -121,6 +127,8 @@ def profile_traffic(kernel_key, shash):
     except Exception:
         return None
     if not d or d.get("source_hash") != shash:
+        return None
+    if d.get("sources") != {f: source_hash(f) for f in HOP_KERNEL_SOURCES}:
         return None
     return d.get("dram_bytes_per_launch")
 
