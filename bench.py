@@ -374,7 +374,7 @@ def hop_variant_label(v, Ls):
         form = "two s-slices per thread, packed FP32" + (", cp.async staging" if v >= 20 else "")
         name = "hop_kernel_pair"
     else:
-        form = ("scalar" if v in (0, 1, 2, 3, 18, 19) else "neighbour prefetch" if v in (4, 5)
+        form = ("scalar" if v in (1, 2, 3, 18, 19, 26) else "neighbour prefetch" if v in (4, 5)
                 else "packed FP32 (re, im)" if v in (6, 7) else "2^4 hypercube tiles" if v in (8, 9)
                 else "y-row CTAs" if 14 <= v <= 17 else "L2 prefetch")
         name = "hop_kernel"

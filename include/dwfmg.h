@@ -147,7 +147,8 @@ int dwf_status(dwf_ctx* ctx, void* stream);
  * 2^4 hypercube tiles, two s-slices per thread with packed FP32 over the
  * pair (loads into registers, or staged in shared memory by cp.async with 2,
  * 4 or 8 neighbours in flight), CTAs of 2 or 4 y-rows, the scalar form
- * with an L2 prefetch of the rows a CTA a wave later reads first; id 0 is the
+ * with an L2 prefetch of the rows a CTA a wave later reads first, the scalar
+ * form without a register cap; id 0 is the
  * untuned choice by lattice size: a kernel that streams the lattice along t
  * through shared memory where that fills the GPU, else the scalar form under
  * 64 registers; DWF_HOP_VARIANTS
@@ -162,7 +163,7 @@ int dwf_status(dwf_ctx* ctx, void* stream);
  * read the choice (0 = untuned default; valid ids 0 .. DWF_HOP_VARIANTS-1;
  * dwf_set_hop_variant returns DWF_EINVAL for a variant that does not tile
  * the lattice). */
-#define DWF_HOP_VARIANTS 26
+#define DWF_HOP_VARIANTS 27
 
 /* Arithmetic of the FP64-precision hopping launches of a context (every
  * DWF_F64 D_hop, M_pc, D_DW and H_DW application, including the FP64

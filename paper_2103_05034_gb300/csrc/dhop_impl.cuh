@@ -852,9 +852,9 @@ constexpr long long HOP_F64_SMALL = 16 * 152;
 // uncapped it takes 143: one M_pc of 16^3x32x16 205 us against 163).  The
 // autotuner (dwf_autotune) times the rest on the context's lattice and keeps
 // the fastest per precision.
-static_assert(DWF_HOP_VARIANTS == 26, "variant table below");
+static_assert(DWF_HOP_VARIANTS == 27, "variant table below");
 __host__ __device__ constexpr int hop_variant_regs(int v) {
-  return v <= 0 ? 0 : v == 1 ? 96 : v == 2 ? 80 : v == 3 ? 64 : v == 4 ? 128 : v == 5 ? 96 : v == 6 ? 64 : v == 7 ? 80
+  return v == 0 ? 0 : v == 1 ? 96 : v == 2 ? 80 : v == 3 ? 64 : v == 4 ? 128 : v == 5 ? 96 : v == 6 ? 64 : v == 7 ? 80
          : v == 8 ? 64 : v == 9 ? 80 : v == 10 ? 128 : v == 11 ? 112 : v == 12 ? 96 : v == 13 ? 0
          : v == 14 ? 64 : v == 15 ? 80 : v == 16 ? 64 : v == 17 ? 80 : v == 18 ? 56 : v == 19 ? 48
          : v == 23 ? 64 : v == 24 ? 64 : v == 25 ? 80 : 0;
@@ -875,7 +875,11 @@ __host__ __device__ constexpr int hop_variant_rows(int v) {
 // (hop_kernel_pair)
 __host__ __device__ constexpr int hop_variant_pf(int v) {
   return v >= 23 ? 0 : v >= 20 ? 4 : v >= 14 ? 0 : v >= 10 ? 4 : v >= 8 ? 3 : v >= 6 ? 2 : v >= 4 ? 1 : 0;
-}  // 18, 19: scalar with 56 / 48 registers; 23-25: scalar with L2 prefetch
+}  // 18, 19: scalar with 56 / 48 registers; 23-25: scalar with L2 prefetch; 26: scalar without a cap
+constexpr int HOP_UNCAPPED = 26;
+static_assert(hop_variant_regs(HOP_UNCAPPED) == 0 && hop_variant_pf(HOP_UNCAPPED) == 0 && hop_variant_rows(HOP_UNCAPPED) == 1 &&
+                  hop_variant_depth(HOP_UNCAPPED) == 0 && hop_variant_l2pf(HOP_UNCAPPED) == 0,
+              "the plain scalar kernel");
 
 // SMs of the current device (0: none).
 inline int device_sms() {
@@ -958,7 +962,7 @@ inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream
     // thread, and nothing waits for a slot.  One hop of a filter, uncapped
     // against 64 registers: 6x10x4x16 Ls 8 7.9 / 9.9 us, 6x6x8x12 Ls 24 10.0 /
     // 12.0; past one round 8^3x16 Ls 16 13.6 / 12.1, four fields 43.5 / 33.8.
-    launch_hop_v<P, LSV, -1>(hp, grid, st);
+    launch_hop_v<P, LSV, HOP_UNCAPPED>(hp, grid, st);
   } else if constexpr (LSV < 16) {
     launch_hop_v<P, LSV, 0>(hp, grid, st);
   } else if constexpr (P == DWF_P_DF) {
@@ -997,6 +1001,7 @@ inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream
       case 23: launch_hop_v<P, LSV, 23>(hp, grid, st); break;
       case 24: launch_hop_v<P, LSV, 24>(hp, grid, st); break;
       case 25: launch_hop_v<P, LSV, 25>(hp, grid, st); break;
+      case HOP_UNCAPPED: launch_hop_v<P, LSV, HOP_UNCAPPED>(hp, grid, st); break;
       default: launch_hop_v<P, LSV, 0>(hp, grid, st); break;
     }
   }
