@@ -162,7 +162,14 @@ int dwf_status(dwf_ctx* ctx, void* stream);
  * before returning; tuning launches are not counted.  Synchronises.  dwf_set_hop_variant / dwf_get_hop_variant pin or
  * read the choice (0 = untuned default; valid ids 0 .. DWF_HOP_VARIANTS-1;
  * dwf_set_hop_variant returns DWF_EINVAL for a variant that does not tile
- * the lattice). */
+ * the lattice).  Where id 0 wins because it streams, the launches that do not
+ * stream (those of the solvers that end in a CG step, those of the filters and
+ * the smoother that end in a Chebyshev step, lattices and fields the streaming
+ * kernel does not fit) take the fastest variant of those that do not, and the
+ * L2 budget of the traversal is tuned on that one.
+ * dwf_set_hop_scalar_variant / dwf_get_hop_scalar_variant set or read it (0:
+ * the untuned choice; dwf_set_hop_variant resets it to 0); it matters only
+ * while the choice itself is 0. */
 #define DWF_HOP_VARIANTS 27
 
 /* Arithmetic of the FP64-precision hopping launches of a context (every
@@ -182,6 +189,8 @@ int dwf_get_f64_arithmetic(const dwf_ctx* ctx);
 int dwf_autotune(dwf_ctx* ctx, int prec, int reps, double* best_ms, void* stream);
 int dwf_set_hop_variant(dwf_ctx* ctx, int prec, int variant);
 int dwf_get_hop_variant(const dwf_ctx* ctx, int prec);
+int dwf_set_hop_scalar_variant(dwf_ctx* ctx, int prec, int variant);
+int dwf_get_hop_scalar_variant(const dwf_ctx* ctx, int prec);
 
 /* ------------------------------------------------------------------ operators */
 

@@ -112,6 +112,8 @@ _SIGS = {
     "dwf_get_f64_arithmetic": (I, [P]),
     "dwf_set_hop_variant": (I, [P, I, I]),
     "dwf_get_hop_variant": (I, [P, I]),
+    "dwf_set_hop_scalar_variant": (I, [P, I, I]),
+    "dwf_get_hop_scalar_variant": (I, [P, I]),
     "dwf_dhop": (I, [P, P, P, I, I, I, I, P]),
     "dwf_mooee": (I, [P, P, P, D, I, I, I, P]),
     "dwf_mooee_inv": (I, [P, P, P, D, I, I, I, P]),

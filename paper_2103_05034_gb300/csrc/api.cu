@@ -350,10 +350,10 @@ int launch_hop(dwf_ctx* c, const HopLaunch& h, int prec, cudaStream_t st, int* n
                                                  : dwf_launch_hop_f64(hp, c->g.Ls, h.nrhs, c->hop_variant[0], st, nblocks);
       break;
     case DWF_F32:
-      rc = dwf_launch_hop_f32(hp, c->g.Ls, h.nrhs, c->hop_variant[1], st, nblocks, &streamed);
+      rc = dwf_launch_hop_f32(hp, c->g.Ls, h.nrhs, c->hop_variant[1], c->hop_scalar[1], st, nblocks, &streamed);
       break;
     case DWF_F16S:
-      rc = dwf_launch_hop_f16(hp, c->g.Ls, h.nrhs, c->hop_variant[2], st, nblocks, &streamed);
+      rc = dwf_launch_hop_f16(hp, c->g.Ls, h.nrhs, c->hop_variant[2], c->hop_scalar[2], st, nblocks, &streamed);
       break;
     default:
       return dwf_fail(c, DWF_EINVAL, "bad precision");
@@ -389,12 +389,103 @@ extern "C" int dwf_set_hop_variant(dwf_ctx* c, int prec, int variant) {
   if (!c || prec < DWF_F64 || prec > DWF_F16S || variant < 0 || variant >= DWF_HOP_VARIANTS) return DWF_EINVAL;
   if (!hop_variant_fits(c, prec, variant)) return dwf_fail(c, DWF_EINVAL, "hop variant does not tile the lattice");
   c->hop_variant[prec] = variant;
+  c->hop_scalar[prec] = 0;
   return DWF_OK;
 }
 
 extern "C" int dwf_get_hop_variant(const dwf_ctx* c, int prec) {
   if (!c || prec < DWF_F64 || prec > DWF_F16S) return DWF_EINVAL;
   return c->hop_variant[prec];
+}
+
+extern "C" int dwf_set_hop_scalar_variant(dwf_ctx* c, int prec, int variant) {
+  if (!c || prec < DWF_F64 || prec > DWF_F16S || variant < 0 || variant >= DWF_HOP_VARIANTS) return DWF_EINVAL;
+  if (!hop_variant_fits(c, prec, variant)) return dwf_fail(c, DWF_EINVAL, "hop variant does not tile the lattice");
+  c->hop_scalar[prec] = variant;
+  return DWF_OK;
+}
+
+extern "C" int dwf_get_hop_scalar_variant(const dwf_ctx* c, int prec) {
+  if (!c || prec < DWF_F64 || prec > DWF_F16S) return DWF_EINVAL;
+  return c->hop_scalar[prec];
+}
+
+// Times `reps` plain D_hop launches of the context's present choice after one
+// to warm up; *streamed: the streaming kernel took them.
+static int time_hop(dwf_ctx* c, void* out, const void* in, int prec, int reps, cudaEvent_t e0, cudaEvent_t e1, float* ms,
+                    bool* streamed, cudaStream_t st) {
+  HopLaunch h;
+  memset(&h, 0, sizeof(h));
+  h.out = out;
+  h.in = in;
+  h.nrhs = 1;
+  h.alpha = 1.0;
+  const int64_t s0 = c->streamed;
+  int rc = launch_hop(c, h, prec, st, nullptr);
+  if (rc) return rc;
+  *streamed = c->streamed != s0;
+  DWF_CUDA(c, cudaEventRecord(e0, st));
+  for (int r = 0; r < reps; r++) {
+    rc = launch_hop(c, h, prec, st, nullptr);
+    if (rc) return rc;
+  }
+  DWF_CUDA(c, cudaEventRecord(e1, st));
+  DWF_CUDA(c, cudaEventSynchronize(e1));
+  DWF_CUDA(c, cudaEventElapsedTime(ms, e0, e1));
+  *ms /= reps;
+  return DWF_OK;
+}
+
+// The choice by time.  Launches that the streaming kernel does not take (those
+// that end in a CG or Chebyshev step above all) are left to the fastest variant
+// that does not stream, and the L2 budget is that of the launches that walk the
+// lattice by it (the streaming kernel does not).
+static int tune_hop(dwf_ctx* c, void* out, const void* in, int prec, int reps, cudaEvent_t e0, cudaEvent_t e1, float* best_ms,
+                    cudaStream_t st) {
+  // FP64: one kernel, or four register caps of the float-float kernel
+  const int nv = c->g.Ls < 16 ? 1 : prec == DWF_F64 ? (c->f64_arith == DWF_ARITH_FLOAT_FLOAT ? 4 : 1) : DWF_HOP_VARIANTS;
+  int best = 0, best_scalar = 0;
+  float t_best = 1e30f, t_scalar = 1e30f;
+  bool best_streams = false;
+  c->hop_scalar[prec] = 0;
+  for (int v = 0; v < nv; v++) {
+    if (!hop_variant_fits(c, prec, v)) continue;
+    c->hop_variant[prec] = v;
+    float ms = 0;
+    bool streamed = false;
+    int rc = time_hop(c, out, in, prec, reps, e0, e1, &ms, &streamed, st);
+    if (rc) return rc;
+    if (ms < t_best) {
+      t_best = ms;
+      best = v;
+      best_streams = streamed;
+    }
+    if (!streamed && ms < t_scalar) {
+      t_scalar = ms;
+      best_scalar = v;
+    }
+  }
+  // then the L2 budget of the z-chunked traversal for the chosen variant
+  c->hop_variant[prec] = best_scalar;
+  const double budgets[5] = {48e6, 16e6, 32e6, 80e6, 120e6};
+  double best_budget = 48e6;
+  for (int bi = 1; bi < 5 && nv > 1; bi++) {
+    c->hop_l2_budget[prec] = budgets[bi];
+    float ms = 0;
+    bool streamed = false;
+    int rc = time_hop(c, out, in, prec, reps, e0, e1, &ms, &streamed, st);
+    if (rc) return rc;
+    if (ms < 0.98f * t_scalar) {  // a clear gain over the default
+      t_scalar = ms;
+      best_budget = budgets[bi];
+    }
+  }
+  c->hop_l2_budget[prec] = best_budget;
+  if (t_scalar < t_best) best_streams = false;
+  c->hop_variant[prec] = best_streams ? best : best_scalar;
+  c->hop_scalar[prec] = best_streams ? best_scalar : 0;
+  *best_ms = best_streams ? t_best : t_scalar;
+  return DWF_OK;
 }
 
 extern "C" int dwf_autotune(dwf_ctx* c, int prec, int reps, double* best_ms, void* stream) {
@@ -408,64 +499,16 @@ extern "C" int dwf_autotune(dwf_ctx* c, int prec, int reps, double* best_ms, voi
   cudaEvent_t e0, e1;
   DWF_CUDA(c, cudaEventCreate(&e0));
   DWF_CUDA(c, cudaEventCreate(&e1));
-  // FP64: one kernel, or four register caps of the float-float kernel
-  const int nv = c->g.Ls < 16 ? 1 : prec == DWF_F64 ? (c->f64_arith == DWF_ARITH_FLOAT_FLOAT ? 4 : 1) : DWF_HOP_VARIANTS;
-  int best = 0;
-  float best_t = 1e30f;
-  const int64_t launches0 = c->launches;
-  const double bytes0 = c->hop_bytes;
-  const int64_t streamed0 = c->streamed;
-  for (int v = 0; v < nv; v++) {
-    if (!hop_variant_fits(c, prec, v)) continue;
-    c->hop_variant[prec] = v;
-    HopLaunch h;
-    memset(&h, 0, sizeof(h));
-    h.out = b;
-    h.in = a;
-    h.out_parity = 0;
-    h.nrhs = 1;
-    h.alpha = 1.0;
-    int rc = launch_hop(c, h, prec, st, nullptr);  // warm-up
-    if (rc) return rc;
-    cudaEventRecord(e0, st);
-    for (int r = 0; r < reps; r++) launch_hop(c, h, prec, st, nullptr);
-    cudaEventRecord(e1, st);
-    DWF_CUDA(c, cudaEventSynchronize(e1));
-    float ms = 0;
-    cudaEventElapsedTime(&ms, e0, e1);
-    ms /= reps;
-    if (ms < best_t) {
-      best_t = ms;
-      best = v;
-    }
+  const int64_t launches0 = c->launches, streamed0 = c->streamed;
+  const double bytes0 = c->hop_bytes, budget0 = c->hop_l2_budget[prec];
+  const int variant0 = c->hop_variant[prec], scalar0 = c->hop_scalar[prec];
+  float best_t = 0;
+  const int rc = tune_hop(c, b, a, prec, reps, e0, e1, &best_t, st);
+  if (rc) {  // the choice stays what it was
+    c->hop_variant[prec] = variant0;
+    c->hop_scalar[prec] = scalar0;
+    c->hop_l2_budget[prec] = budget0;
   }
-  // then the L2 budget of the z-chunked traversal for the chosen variant
-  c->hop_variant[prec] = best;
-  const double budgets[5] = {48e6, 16e6, 32e6, 80e6, 120e6};
-  double best_budget = 48e6;
-  for (int bi = 1; bi < 5 && nv > 1; bi++) {
-    c->hop_l2_budget[prec] = budgets[bi];
-    HopLaunch h;
-    memset(&h, 0, sizeof(h));
-    h.out = b;
-    h.in = a;
-    h.nrhs = 1;
-    h.alpha = 1.0;
-    int rc = launch_hop(c, h, prec, st, nullptr);
-    if (rc) return rc;
-    cudaEventRecord(e0, st);
-    for (int r = 0; r < reps; r++) launch_hop(c, h, prec, st, nullptr);
-    cudaEventRecord(e1, st);
-    DWF_CUDA(c, cudaEventSynchronize(e1));
-    float ms = 0;
-    cudaEventElapsedTime(&ms, e0, e1);
-    ms /= reps;
-    if (ms < 0.98f * best_t) {  // a clear gain over the default
-      best_t = ms;
-      best_budget = budgets[bi];
-    }
-  }
-  c->hop_l2_budget[prec] = best_budget;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   c->launches = launches0;  // tuning launches are not counted
@@ -478,6 +521,7 @@ extern "C" int dwf_autotune(dwf_ctx* c, int prec, int reps, double* best_ms, voi
     c->ws[slot] = nullptr;
     c->ws_bytes[slot] = 0;
   }
+  if (rc) return rc;
   if (best_ms) *best_ms = best_t;
   DWF_CUDA(c, cudaGetLastError());
   return dwf_wait_status(c);

@@ -4,5 +4,5 @@
 #include "dfloat.cuh"
 
 int dwf_launch_hop_df(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb) {
-  return dwfk::launch_hop_prec<DWF_P_DF>(hp, Ls, nrhs, variant, st, nb);
+  return dwfk::launch_hop_prec<DWF_P_DF>(hp, Ls, nrhs, variant, variant, st, nb, nullptr);
 }

@@ -1,9 +1,9 @@
 // Hopping-term and site-local fifth-dimension kernels instantiated for DWF_F16S.
 #include "dhop_impl.cuh"
 
-int dwf_launch_hop_f16(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb,
+int dwf_launch_hop_f16(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, int scalar, cudaStream_t st, int* nb,
                        bool* streamed) {
-  return dwfk::launch_hop_prec<DWF_F16S>(hp, Ls, nrhs, variant, st, nb, streamed);
+  return dwfk::launch_hop_prec<DWF_F16S>(hp, Ls, nrhs, variant, scalar, st, nb, streamed);
 }
 
 int dwf_launch_mooee_f16(void* out, const void* in, const dwfk::HopParams& hp, int dagger,

@@ -3,7 +3,7 @@
 
 int dwf_launch_hop_f64(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st,
                        int* nb) {
-  return dwfk::launch_hop_prec<DWF_F64>(hp, Ls, nrhs, variant, st, nb);
+  return dwfk::launch_hop_prec<DWF_F64>(hp, Ls, nrhs, variant, variant, st, nb, nullptr);
 }
 
 int dwf_launch_mooee_f64(void* out, const void* in, const dwfk::HopParams& hp, int dagger,

@@ -1135,58 +1135,54 @@ inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, in
 }
 
 // The streaming kernel, where a plain launch of this shape has one.
-template <int P>
-bool try_hop_stream(const HopParams& hp, int Ls, int nrhs, cudaStream_t st, int* nblocks) {
-  if constexpr (P == DWF_F32 || P == DWF_F16S) {
-    if (hp.cheb_mode || hp.cg_mode) return false;
-    if (Ls == 8) return launch_hop_stream<P, 8, 6>(hp, nrhs, st, nblocks);
-    if constexpr (P == DWF_F32) {
-      if (Ls == 16)
-        return launch_hop_stream<P, 16, 4>(hp, nrhs, st, nblocks) || launch_hop_stream<P, 16, 3>(hp, nrhs, st, nblocks);
-      if (Ls == 24) return launch_hop_stream<P, 24, 2>(hp, nrhs, st, nblocks);
-    }
-  }
+template <int P, int LSV>
+bool try_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, int* nblocks) {
+  if (hp.cheb_mode || hp.cg_mode) return false;
+  if constexpr ((P == DWF_F32 || P == DWF_F16S) && LSV == 8) return launch_hop_stream<P, 8, 6>(hp, nrhs, st, nblocks);
+  if constexpr (P == DWF_F32 && LSV == 16)
+    return launch_hop_stream<P, 16, 4>(hp, nrhs, st, nblocks) || launch_hop_stream<P, 16, 3>(hp, nrhs, st, nblocks);
+  if constexpr (P == DWF_F32 && LSV == 24) return launch_hop_stream<P, 24, 2>(hp, nrhs, st, nblocks);
   return false;
 }
 
+// A launch at Ls = LSV: variant 0 streams where its rule says so; a launch that
+// it does not take runs variant `scalar` (0: the untuned choice of launch_hop_ls).
+template <int P, int LSV>
+int launch_hop_at(const HopParams& hp, int nrhs, int variant, int scalar, cudaStream_t st, int* nblocks, bool* streamed) {
+  if (variant == 0) {
+    if (try_hop_stream<P, LSV>(hp, nrhs, st, nblocks)) {
+      if (streamed) *streamed = true;
+      return DWF_OK;
+    }
+    variant = scalar;
+  }
+  constexpr int SB = HopShape<LSV>::SB;
+  const int ry = (P == DWF_F64 || P == DWF_P_DF || LSV < 16) ? 1 : hop_variant_rows(variant);
+  if (ry > 1 && (hp.Lxh % SB || hp.L1 % ry)) return DWF_EINVAL;
+  dim3 grid((hp.Vh + SB * ry - 1) / (SB * ry), nrhs, 1);
+  if constexpr (P == DWF_F64) {
+    if ((long long)hp.Vh * LSV * nrhs <= HOP_F64_DIRS) {
+      grid.x = (hp.Vh + DirsCfg<LSV>::SITES - 1) / DirsCfg<LSV>::SITES;
+      if (nblocks) *nblocks = grid.x * grid.y;
+      hop_dirs_f64<LSV><<<grid, DirsCfg<LSV>::NT, 0, st>>>(hp);
+      return DWF_OK;
+    }
+    if ((long long)grid.x * nrhs < HOP_F64_SMALL) grid.x = (hp.Vh + HopShape<LSV>::SB1 - 1) / HopShape<LSV>::SB1;
+  }
+  if (nblocks) *nblocks = grid.x * grid.y;
+  return launch_hop_ls<P, LSV>(hp, grid, variant, st);
+}
+
 template <int P>
-int launch_hop_prec(const HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nblocks,
-                    bool* streamed = nullptr) {
-  if (variant == 0 && try_hop_stream<P>(hp, Ls, nrhs, st, nblocks)) {
-    if (streamed) *streamed = true;
-    return DWF_OK;
-  }
-  dim3 grid;
-  grid.y = nrhs;
-  grid.z = 1;
-#define DWF_HOP_CASE(LSV)                                                        \
-  case LSV: {                                                                    \
-    constexpr int SB = HopShape<LSV>::SB;                                        \
-    const int ry = (P == DWF_F64 || P == DWF_P_DF || LSV < 16) ? 1 : hop_variant_rows(variant); \
-    if (ry > 1 && (hp.Lxh % SB || hp.L1 % ry)) return DWF_EINVAL;                \
-    grid.x = (hp.Vh + SB * ry - 1) / (SB * ry);                                  \
-    if constexpr (P == DWF_F64) {                                                \
-      if ((long long)hp.Vh * LSV * nrhs <= HOP_F64_DIRS) {                       \
-        grid.x = (hp.Vh + DirsCfg<LSV>::SITES - 1) / DirsCfg<LSV>::SITES;        \
-        if (nblocks) *nblocks = grid.x * grid.y;                                 \
-        hop_dirs_f64<LSV><<<grid, DirsCfg<LSV>::NT, 0, st>>>(hp);                \
-        return DWF_OK;                                                           \
-      }                                                                          \
-      if ((long long)grid.x * nrhs < HOP_F64_SMALL)                              \
-        grid.x = (hp.Vh + HopShape<LSV>::SB1 - 1) / HopShape<LSV>::SB1;          \
-    }                                                                            \
-    if (nblocks) *nblocks = grid.x * grid.y;                                     \
-    return launch_hop_ls<P, LSV>(hp, grid, variant, st);                         \
-  }
+int launch_hop_prec(const HopParams& hp, int Ls, int nrhs, int variant, int scalar, cudaStream_t st, int* nblocks,
+                    bool* streamed) {
   switch (Ls) {
-    DWF_HOP_CASE(4)
-    DWF_HOP_CASE(8)
-    DWF_HOP_CASE(16)
-    DWF_HOP_CASE(24)
-    default:
-      return DWF_EINVAL;
+    case 4: return launch_hop_at<P, 4>(hp, nrhs, variant, scalar, st, nblocks, streamed);
+    case 8: return launch_hop_at<P, 8>(hp, nrhs, variant, scalar, st, nblocks, streamed);
+    case 16: return launch_hop_at<P, 16>(hp, nrhs, variant, scalar, st, nblocks, streamed);
+    case 24: return launch_hop_at<P, 24>(hp, nrhs, variant, scalar, st, nblocks, streamed);
+    default: return DWF_EINVAL;
   }
-#undef DWF_HOP_CASE
 }
 
 template <int P>
@@ -1216,9 +1212,11 @@ int launch_mooee_prec(void* out, const void* in, const HopParams& hp, int dagger
 
 // Per-precision entry points (defined in dhop_f64.cu, dhop_f32.cu, dhop_f16.cu).
 int dwf_launch_hop_f64(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb);
-// (*streamed: the streaming kernel took the launch)
-int dwf_launch_hop_f32(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb, bool* streamed);
-int dwf_launch_hop_f16(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb, bool* streamed);
+// (scalar: the variant where 0 does not stream; *streamed: the streaming kernel took the launch)
+int dwf_launch_hop_f32(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, int scalar, cudaStream_t st, int* nb,
+                       bool* streamed);
+int dwf_launch_hop_f16(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, int scalar, cudaStream_t st, int* nb,
+                       bool* streamed);
 // FP64 storage, float-float arithmetic (dhop_df.cu)
 int dwf_launch_hop_df(const dwfk::HopParams& hp, int Ls, int nrhs, int variant, cudaStream_t st, int* nb);
 int dwf_launch_mooee_f64(void* out, const void* in, const dwfk::HopParams& hp, int dagger,

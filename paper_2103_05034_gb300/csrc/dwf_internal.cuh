@@ -130,6 +130,7 @@ struct dwf_ctx {
   double* hscal;      // pinned host mirror
   int* wait_flag;     // behind hscal (a clone's: its source's): set by a kernel whose bounded wait gave up
   int hop_variant[3]; // tuned hopping-kernel variant per precision
+  int hop_scalar[3];  // where that is 0: the variant of the launches that do not stream
   int f64_arith;      // FP64 hopping launches: DWF_ARITH_FP64 or DWF_ARITH_FLOAT_FLOAT
   double hop_l2_budget[3];  // L2 bytes the z-chunked traversal plans for (0: 48 MB)
   int64_t launches;   // kernel launches since the last counter reset

@@ -524,3 +524,12 @@ def dwf_autotune(ctx, prec=F32, reps=20):
 
 def dwf_set_hop_variant(ctx, prec, variant):
     check(lib().dwf_set_hop_variant(ctx.h, prec, variant), ctx.h)
+
+
+def dwf_set_hop_scalar_variant(ctx, prec, variant):
+    """Variant of the launches that choice 0 does not stream."""
+    check(lib().dwf_set_hop_scalar_variant(ctx.h, prec, variant), ctx.h)
+
+
+def dwf_get_hop_scalar_variant(ctx, prec):
+    return lib().dwf_get_hop_scalar_variant(ctx.h, prec)

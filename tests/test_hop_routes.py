@@ -1,0 +1,144 @@
+"""Which kernel a hopping launch runs, without a GPU: the launcher of
+csrc/dhop_impl.cuh linked against a stand-in for the CUDA runtime that records
+the kernel and the grid instead of launching."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_2103_05034_gb300 import build
+
+RUNTIME = r"""
+#include <cstring>
+#include <cuda.h>
+#include <cuda_runtime_api.h>
+
+const void* kernel = nullptr;
+int grid = 0, streams = 0;
+
+static CUresult fake_encode(CUtensorMap* m, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                            const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                            CUtensorMapL2promotion, CUtensorMapFloatOOBfill) {
+  std::memset(m, 0, sizeof(*m));
+  return CUDA_SUCCESS;
+}
+
+extern "C" {
+cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 152; return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, int, size_t) { *n = 4; return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) {
+  *n = 4;
+  return cudaSuccess;
+}
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult*) {
+  *f = (void*)fake_encode;
+  return cudaSuccess;
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+  kernel = f;
+  grid = c->gridDim.x;
+  streams++;
+  return cudaSuccess;
+}
+cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) { *k = (cudaKernel_t)f; return cudaSuccess; }
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3, void**, size_t, cudaStream_t) {
+  kernel = (const void*)k;
+  grid = g.x;
+  return cudaSuccess;
+}
+}
+"""
+
+# the launch's route; Route::kernel compares with that of another launch
+COMMON = r"""
+#include <cstdio>
+#include <cstring>
+#include "dhop_impl.cuh"
+
+extern const void* kernel;
+extern int grid, streams;
+
+struct Route {
+  const void* kernel;
+  int grid;
+  bool streamed;
+  bool operator==(const Route& o) const { return kernel == o.kernel && grid == o.grid && streamed == o.streamed; }
+};
+
+template <int P, int LS>
+Route route(int x, int y, int z, int t, int nrhs, int variant, int scalar, bool cheb = false) {
+  dwfk::HopParams hp;
+  std::memset(&hp, 0, sizeof(hp));
+  hp.L0 = x;
+  hp.L1 = y;
+  hp.L2 = hp.zc = z;
+  hp.L3 = t;
+  hp.Lxh = x / 2;
+  hp.Vh = x * y * z * t / 2;
+  hp.d = 3.2;
+  hp.rhs_stride = (long long)hp.Vh * 12 * LS;
+  hp.cheb_mode = cheb;
+  kernel = nullptr;
+  grid = streams = 0;
+  bool s = false;
+  const int rc = dwfk::launch_hop_at<P, LS>(hp, nrhs, variant, scalar, nullptr, nullptr, &s);
+  if (rc || !kernel || s != (streams == 1)) std::printf("launch failed\n");
+  return {kernel, grid, s};
+}
+static int bad = 0;
+#define CHECK(c)                              \
+  if (!(c)) {                                 \
+    std::printf("line %d: %s\n", __LINE__, #c); \
+    bad++;                                    \
+  }
+"""
+
+SCALAR = COMMON + r"""
+int main() {
+  // 16^3x32 streams; its Chebyshev launches take the scalar variant
+  const auto r = [](int variant, int scalar, bool cheb) { return route<DWF_F32, 16>(16, 16, 16, 32, 1, variant, scalar, cheb); };
+  CHECK(r(0, 0, false).streamed && r(0, 16, false).streamed);
+  CHECK(!r(0, 0, true).streamed);
+  for (int v = 1; v < DWF_HOP_VARIANTS; v++) {
+    CHECK(!r(v, 0, false).streamed);
+    CHECK(r(0, v, true) == r(v, 0, true));
+    CHECK(r(v, 5, true) == r(v, 0, true));  // a choice other than 0 is everybody's
+  }
+  CHECK(r(0, 16, true).grid == 16 * 16 * 16 * 32 / 2 / 32);  // CTAs of eight sites on four rows
+  CHECK(!(r(0, 16, true) == r(0, 3, true)));
+  // a lattice that does not stream takes it for every launch
+  CHECK(!(route<DWF_F32, 16>(16, 4, 4, 4, 1, 0, 0).streamed));
+  CHECK((route<DWF_F32, 16>(16, 4, 4, 4, 1, 0, 26) == route<DWF_F32, 16>(16, 4, 4, 4, 1, 26, 0)));
+  std::printf("bad %d\n", bad);
+  return bad != 0;
+}
+"""
+
+
+def _run(tmp_path, program):
+    try:
+        nvcc = build.nvcc()
+    except RuntimeError:
+        pytest.skip("no nvcc")
+    if shutil.which("g++") is None:
+        pytest.skip("no host compiler")
+    (tmp_path / "program.cu").write_text(program)
+    (tmp_path / "runtime.cpp").write_text(RUNTIME)
+    exe = tmp_path / "routes"
+    # the host side is what runs: device code only as far as PTX
+    subprocess.run([nvcc, "-gencode", "arch=compute_103a,code=compute_103a", "-std=c++17", "-O1", "--expt-relaxed-constexpr",
+                    "-cudart", "shared", "-I", build.CSRC, str(tmp_path / "program.cu"), str(tmp_path / "runtime.cpp"),
+                    "-o", str(exe)], check=True, capture_output=True)
+    env = dict(os.environ)
+    env["LD_LIBRARY_PATH"] = os.path.join(os.path.dirname(os.path.dirname(nvcc)), "lib64") + ":" + env.get("LD_LIBRARY_PATH", "")
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60, env=env)
+    assert r.returncode == 0 and r.stdout.strip() == "bad 0", r.stdout + r.stderr
+
+
+def test_launches_that_do_not_stream_take_the_scalar_choice(tmp_path):
+    _run(tmp_path, SCALAR)
