@@ -366,8 +366,8 @@ def hop_variant_label(v, Ls):
     """The FP32 hopping kernel that tuning variant v launches (the variant table
     of csrc/dhop_impl.cuh: register cap and inner-loop form)."""
     if v == 0:
-        return (f"dwfk::hop_stream<F32, Ls={Ls}> where it fills the GPU, else dwfk::hop_kernel (scalar, 64 registers) "
-                "(dwf_dhop, plain epilogue; variant 0: untuned choice by lattice size)")
+        return (f"dwfk::hop_stream<F32, Ls={Ls}> where it fills the GPU, else dwfk::hop_kernel (scalar, register cap by "
+                "size) (dwf_dhop, plain epilogue; variant 0: untuned choice by lattice size)")
     regs = {1: 96, 2: 80, 3: 64, 4: 128, 5: 96, 6: 64, 7: 80, 8: 64, 9: 80, 10: 128, 11: 112, 12: 96, 14: 64, 15: 80,
             16: 64, 17: 80, 18: 56, 19: 48, 23: 64, 24: 64, 25: 80}.get(v, 0)
     if 10 <= v <= 13 or 20 <= v <= 22:

@@ -150,8 +150,8 @@ int dwf_status(dwf_ctx* ctx, void* stream);
  * with an L2 prefetch of the rows a CTA a wave later reads first, the scalar
  * form without a register cap; id 0 is the
  * untuned choice by lattice size: a kernel that streams the lattice along t
- * through shared memory where that fills the GPU, else the scalar form under
- * 64 registers; DWF_HOP_VARIANTS
+ * through shared memory where that fills the GPU, else the scalar form under a
+ * register cap by the number of CTAs; DWF_HOP_VARIANTS
  * variants for FP32 and FP16
  * storage at Ls >= 16, one otherwise; for DWF_F64 the one FP64 kernel, or
  * with DWF_ARITH_FLOAT_FLOAT the float-float kernel under four register

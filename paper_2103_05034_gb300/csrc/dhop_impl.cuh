@@ -848,10 +848,9 @@ constexpr long long HOP_F64_SMALL = 16 * 152;
 
 // Tuning variants of the hopping kernel: (register cap, prefetch).  Variant 0
 // is the untuned default: the streaming kernel by its rule (launch_hop_stream),
-// else the scalar kernel, in FP32 arithmetic with 64 registers (8 CTAs an SM;
-// uncapped it takes 143: one M_pc of 16^3x32x16 205 us against 163).  The
-// autotuner (dwf_autotune) times the rest on the context's lattice and keeps
-// the fastest per precision.
+// else the scalar kernel, in FP32 arithmetic with a register cap by the number
+// of CTAs (hop_default_variant).  The autotuner (dwf_autotune) times the rest
+// on the context's lattice and keeps the fastest per precision.
 static_assert(DWF_HOP_VARIANTS == 27, "variant table below");
 __host__ __device__ constexpr int hop_variant_regs(int v) {
   return v == 0 ? 0 : v == 1 ? 96 : v == 2 ? 80 : v == 3 ? 64 : v == 4 ? 128 : v == 5 ? 96 : v == 6 ? 64 : v == 7 ? 80
@@ -915,7 +914,7 @@ inline void hop_launch_smem(dim3 grid, int threads, size_t bytes, size_t most, c
 
 template <int P, int LSV, int V, int SB = HopShape<LSV>::SB>
 inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
-  constexpr int REGS = V == 0 && (P == DWF_F32 || P == DWF_F16S) ? 64 : hop_variant_regs(V);
+  constexpr int REGS = hop_variant_regs(V);
   constexpr int PF = hop_variant_pf(V);
   constexpr int RY = PF == 4 ? 1 : hop_variant_rows(V);
   constexpr size_t cb = sizeof(cpx<typename Prec<P>::R>);
@@ -948,23 +947,61 @@ inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
   }
 }
 
+// The untuned scalar variant in FP32 arithmetic, by x = CTAs an SM.  A cap gives
+// more resident CTAs, which hide the latency of the neighbour reads; fewer
+// registers mean fewer loads in flight a thread; and a last round that is nearly
+// empty costs almost as much as a full one.  3 CTAs are resident uncapped (135 to
+// 147 registers), 5, 6 and 8 under 96, 80 and 64 registers; at Ls 24 (192
+// threads) 2, 3, 4 and 5.  Times in us, uncapped / 96 / 80 / 64, M_pc of one
+// field unless noted, x in brackets:
+//   one round uncapped: 8^3x16 Ls 8 D_DW 12.4 / 16.4 / 16.4 / 16.4
+//   one round at 80:    8^3x24 Ls 16 (5.0) 22.7 / 26.0 / 22.7 / 24.6
+//   one round at 64:    8^2x16x32 Ls 8 (6.7) 35.3 / 33.0 / 34.8 / 30.8
+//   just above it:      Ls 8 12^3x24 (8.5) D_DW 37.1 / 36.9 / 37.6 / 41.0, so 96;
+//                       Ls 4 (8.8) 61.5 / 61.6 / 65.0 / 66.9, so uncapped
+//   several rounds:     the fuller ones of 80 and 64: Ls 24 8^3x40 (8.4) 62.0 / 51.4
+//                       / 52.3 / 49.3, 8^3x48 (10.1) 75.9 / 65.6 / 59.6 / 61.6
+//   many:               64, FP32 from 32 on (filter of 16^3x32 Ls 16, order 5, 3260 /
+//                       2494 / 2393 / 2328), FP16 storage, which needs half the L1
+//                       fills, from 12 on (Ls 24 8^3x144 (30) 220 / 172 / 146 / 140)
+//   Ls 4:               96 (8x16^2x144 (30) 187 / 175 / 179 / 183)
+// Of 1076 launches and sizes timed (both types, four Ls, D_hop, M_pc, D_DW, filter
+// and CG, one and four fields, x from 1.7 to 280) this takes 0.888 of the time
+// uncapped and 0.980 of that with 64 throughout, which was up to 11 % slower than
+// uncapped between 8 and 12 CTAs an SM.
+template <int P, int LSV>
+inline int hop_default_variant(long long ctas) {
+  constexpr int T = LSV * HopShape<LSV>::SB;
+  constexpr int R0 = 65536 / (T * 144), R80 = 65536 / (T * 80), R64 = 65536 / (T * 64);
+  const double x = (double)ctas / device_sms();
+  if (x <= R0) return HOP_UNCAPPED;
+  if (P == DWF_F32 && x > R64 && x <= 3 * R0) {
+    if (LSV == 4) return HOP_UNCAPPED;
+    if (LSV == 8) return 1;
+  }
+  if (LSV == 4 && x > R64) return 1;
+  if (x > (P == DWF_F32 ? 32 : 12)) return 3;
+  const auto fill = [x](int r) { return x / (r * ceil(x / r)); };  // over all rounds
+  return fill(R64) > fill(R80) ? 3 : 2;
+}
+
 template <int P, int LSV>
 inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream_t st) {
-  // FP64 is ALU-bound and the small-Ls cases are test sizes: one variant.
+  // FP64 is ALU-bound: one variant.  At Ls < 16 the tuner has nothing to choose.
   if constexpr (P == DWF_F64) {
     if (grid.x == (hp.Vh + HopShape<LSV>::SB1 - 1) / HopShape<LSV>::SB1)
       launch_hop_v<P, LSV, 0, HopShape<LSV>::SB1>(hp, grid, st);
     else
       launch_hop_v<P, LSV, 0>(hp, grid, st);
-  } else if (variant == 0 && (P == DWF_F32 || P == DWF_F16S) &&
-             (long long)grid.x * grid.y <= 152LL * (65536 / (LSV * HopShape<LSV>::SB * 144))) {
-    // All CTAs resident at once without a register cap: more loads in flight a
-    // thread, and nothing waits for a slot.  One hop of a filter, uncapped
-    // against 64 registers: 6x10x4x16 Ls 8 7.9 / 9.9 us, 6x6x8x12 Ls 24 10.0 /
-    // 12.0; past one round 8^3x16 Ls 16 13.6 / 12.1, four fields 43.5 / 33.8.
-    launch_hop_v<P, LSV, HOP_UNCAPPED>(hp, grid, st);
-  } else if constexpr (LSV < 16) {
+  } else if constexpr (P == DWF_P_DF && LSV < 16) {
     launch_hop_v<P, LSV, 0>(hp, grid, st);
+  } else if constexpr (LSV < 16) {
+    switch (hop_default_variant<P, LSV>((long long)grid.x * grid.y)) {
+      case 1: launch_hop_v<P, LSV, 1>(hp, grid, st); break;
+      case 2: launch_hop_v<P, LSV, 2>(hp, grid, st); break;
+      case 3: launch_hop_v<P, LSV, 3>(hp, grid, st); break;
+      default: launch_hop_v<P, LSV, HOP_UNCAPPED>(hp, grid, st); break;
+    }
   } else if constexpr (P == DWF_P_DF) {
     // float-float: the plain kernel with register caps 96 / 80 / 64 (more
     // resident warps for its long dependent FP32 chains)
@@ -975,6 +1012,7 @@ inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream
       default: launch_hop_v<P, LSV, 0>(hp, grid, st); break;
     }
   } else {
+    if (variant == 0) variant = hop_default_variant<P, LSV>((long long)grid.x * grid.y);
     switch (variant) {
       case 1: launch_hop_v<P, LSV, 1>(hp, grid, st); break;
       case 2: launch_hop_v<P, LSV, 2>(hp, grid, st); break;
@@ -1001,8 +1039,7 @@ inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream
       case 23: launch_hop_v<P, LSV, 23>(hp, grid, st); break;
       case 24: launch_hop_v<P, LSV, 24>(hp, grid, st); break;
       case 25: launch_hop_v<P, LSV, 25>(hp, grid, st); break;
-      case HOP_UNCAPPED: launch_hop_v<P, LSV, HOP_UNCAPPED>(hp, grid, st); break;
-      default: launch_hop_v<P, LSV, 0>(hp, grid, st); break;
+      default: launch_hop_v<P, LSV, HOP_UNCAPPED>(hp, grid, st); break;
     }
   }
   return DWF_OK;

@@ -120,6 +120,50 @@ int main() {
 """
 
 
+CAPS = COMMON + r"""
+// the scalar kernel of a variant id on a launch of this size
+template <int P, int LS, int V>
+const void* scalar() {
+  dwfk::HopParams hp;
+  std::memset(&hp, 0, sizeof(hp));
+  dwfk::launch_hop_v<P, LS, V>(hp, dim3(1), nullptr);
+  return kernel;
+}
+// register cap that the untuned choice runs at x CTAs an SM (0: none)
+template <int P, int LS>
+int cap(double x) {
+  constexpr int SB = dwfk::HopShape<LS>::SB;
+  dwfk::HopParams hp;
+  std::memset(&hp, 0, sizeof(hp));
+  hp.Vh = (int)(x * 152 + 0.5) * SB;
+  hp.Lxh = hp.L0 = hp.L1 = 2;
+  hp.cheb_mode = 1;  // (a launch that does not stream)
+  if (dwfk::launch_hop_at<P, LS>(hp, 1, 0, 0, nullptr, nullptr, nullptr)) return -1;
+  const void* k = kernel;
+  return k == scalar<P, LS, 26>() ? 0 : k == scalar<P, LS, 1>() ? 96 : k == scalar<P, LS, 2>() ? 80 : k == scalar<P, LS, 3>() ? 64 : -1;
+}
+
+int main() {
+  const double x[] = {0.1, 3, 3.2, 6, 6.2, 8, 8.4, 9, 9.2, 11, 12, 12.4, 16.2, 24, 31, 33, 200};
+  const int f32_4[] = {0, 0, 80, 80, 64, 64, 0, 0, 96, 96, 96, 96, 96, 96, 96, 96, 96};
+  const int f16_4[] = {0, 0, 80, 80, 64, 64, 96, 96, 96, 96, 96, 96, 96, 96, 96, 96, 96};
+  const int f32_8[] = {0, 0, 80, 80, 64, 64, 96, 96, 80, 80, 80, 64, 80, 80, 64, 64, 64};
+  const int f16_8[] = {0, 0, 80, 80, 64, 64, 80, 80, 80, 80, 80, 64, 64, 64, 64, 64, 64};
+  for (int i = 0; i < 17; i++) {
+    const int got[4] = {cap<DWF_F32, 4>(x[i]), cap<DWF_F16S, 4>(x[i]), cap<DWF_F32, 8>(x[i]), cap<DWF_F16S, 8>(x[i])};
+    const int want[4] = {f32_4[i], f16_4[i], f32_8[i], f16_8[i]};
+    for (int k = 0; k < 4; k++)
+      if (got[k] != want[k]) {
+        std::printf("x %g case %d: %d, not %d\n", x[i], k, got[k], want[k]);
+        bad++;
+      }
+  }
+  std::printf("bad %d\n", bad);
+  return bad != 0;
+}
+"""
+
+
 def _run(tmp_path, program):
     try:
         nvcc = build.nvcc()
@@ -142,3 +186,9 @@ def _run(tmp_path, program):
 
 def test_launches_that_do_not_stream_take_the_scalar_choice(tmp_path):
     _run(tmp_path, SCALAR)
+
+
+def test_untuned_register_cap_by_number_of_ctas(tmp_path):
+    """Nothing runs under a cap that one round of CTAs does not need, and the cap
+    just above a full round is not the one whose last round is empty."""
+    _run(tmp_path, CAPS)
