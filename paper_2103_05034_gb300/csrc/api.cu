@@ -124,6 +124,7 @@ extern "C" int dwf_ctx_create(dwf_ctx** out, const int L[4], int Ls, double M5, 
   c->g.Ls = Ls;
   c->M5 = M5;
   cudaGetDevice(&c->device);
+  cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   cudaStream_t st = (cudaStream_t)stream;
   const size_t glinks = (size_t)V4 * 4 * 9;
   const void* Ud = gauge;
@@ -184,6 +185,7 @@ int dwf_ctx_clone_ls(const dwf_ctx* src, int ls, dwf_ctx** out, cudaStream_t st)
   c->g.Ls = ls;
   c->M5 = src->M5;
   c->device = src->device;
+  c->sms = src->sms;
   int rc = DWF_OK;
   const size_t lb = (size_t)c->g.Vh * 72;
   for (int p = 0; p < 2 && rc == DWF_OK; p++) {
@@ -286,6 +288,7 @@ int launch_hop(dwf_ctx* c, const HopLaunch& h, int prec, cudaStream_t st, int* n
   hp.L3 = c->g.L[3];
   hp.Lxh = c->g.Lxh;
   hp.Vh = (int)c->g.Vh;
+  hp.sms = c->sms;
   {
     // z-chunk: the largest even divisor of Lz whose input slab (zc planes of
     // one time slice, over the t-1, t, t+1 slices plus the output) stays

@@ -44,6 +44,7 @@ struct HopParams {
   int zc;  // traversal z-chunk (even divisor of L2; L2 = lexicographic order)
   int l2pf; // > 0: each CTA prefetches into L2 the input rows first read by the
             // CTA l2pf positions later in the traversal (scalar kernel only)
+  int sms;        // of the device (host side of the launch only; 0: ask)
   int* wait_err;  // host-mapped flag raised by a bounded wait that gave up (streaming kernel)
   int out_parity;
   float sg;  // +1: D_hop, -1: D_hop^dag
@@ -894,6 +895,8 @@ inline int device_sms() {
   return n ? *n : ask();
 }
 
+inline int hop_sms(const HopParams& hp) { return hp.sms > 0 ? hp.sms : device_sms(); }
+
 // Dynamic shared memory of one launch: links (SBC*72 complex, twice for the
 // (re,re,-im,im) packed form), or the M_ee^-1 stage (SBC*12*(LS+1) complex)
 // when the epilogue inverts; above 48 KB every device is opted in, once per
@@ -970,10 +973,10 @@ inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
 // uncapped and 0.980 of that with 64 throughout, which was up to 11 % slower than
 // uncapped between 8 and 12 CTAs an SM.
 template <int P, int LSV>
-inline int hop_default_variant(long long ctas) {
+inline int hop_default_variant(long long ctas, int sms) {
   constexpr int T = LSV * HopShape<LSV>::SB;
   constexpr int R0 = 65536 / (T * 144), R80 = 65536 / (T * 80), R64 = 65536 / (T * 64);
-  const double x = (double)ctas / device_sms();
+  const double x = (double)ctas / sms;
   if (x <= R0) return HOP_UNCAPPED;
   if (P == DWF_F32 && x > R64 && x <= 3 * R0) {
     if (LSV == 4) return HOP_UNCAPPED;
@@ -996,7 +999,7 @@ inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream
   } else if constexpr (P == DWF_P_DF && LSV < 16) {
     launch_hop_v<P, LSV, 0>(hp, grid, st);
   } else if constexpr (LSV < 16) {
-    switch (hop_default_variant<P, LSV>((long long)grid.x * grid.y)) {
+    switch (hop_default_variant<P, LSV>((long long)grid.x * grid.y, hop_sms(hp))) {
       case 1: launch_hop_v<P, LSV, 1>(hp, grid, st); break;
       case 2: launch_hop_v<P, LSV, 2>(hp, grid, st); break;
       case 3: launch_hop_v<P, LSV, 3>(hp, grid, st); break;
@@ -1012,7 +1015,7 @@ inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream
       default: launch_hop_v<P, LSV, 0>(hp, grid, st); break;
     }
   } else {
-    if (variant == 0) variant = hop_default_variant<P, LSV>((long long)grid.x * grid.y);
+    if (variant == 0) variant = hop_default_variant<P, LSV>((long long)grid.x * grid.y, hop_sms(hp));
     switch (variant) {
       case 1: launch_hop_v<P, LSV, 1>(hp, grid, st); break;
       case 2: launch_hop_v<P, LSV, 2>(hp, grid, st); break;
@@ -1120,6 +1123,9 @@ inline bool stream_grid(StreamGrid& g, const HopParams& hp, int nrhs, int SX, in
 template <int P, int LS, int SX>
 inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, int* nblocks) {
   typedef StreamCfg<P, LS, SX> C;
+  // fewer than three steps a CTA: not worth the count below, nor asking the runtime
+  const auto too_small = [&](int sms) { return (double)hp.Vh * nrhs < stream_min_fill<P, LS>() * sms * 5 * C::SITES; };
+  if (too_small(hp.sms)) return false;
   static PerDevice<int> cache;  // SMs of a device that has opted in to the shared memory, else 0
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
@@ -1131,8 +1137,7 @@ inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, in
     return device_sms();
   });
   const int sms = ready ? *ready : 0;
-  // fewer than three steps a CTA: not worth the count below
-  if (sms < 1 || (double)hp.Vh * nrhs < stream_min_fill<P, LS>() * sms * 5 * C::SITES) return false;
+  if (sms < 1 || too_small(sms)) return false;
   if (hp.inv_mode && !hp.one_sweep) return false;
   StreamGrid g;
   int grid;

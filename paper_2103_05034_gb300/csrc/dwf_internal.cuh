@@ -117,6 +117,7 @@ struct dwf_ctx {
   Geom g;
   double M5;
   int device;
+  int sms;    // of that device
   // parity-split, double-stored links: links[p] is [Vh][8][3][3] complex,
   // slot 2mu = U_mu(x), slot 2mu+1 = U_mu(x-mu)^dag, for sites x of parity p.
   double2* links64[2];
