@@ -844,8 +844,21 @@ struct HopShape {
 // HOP_F64_SMALL CTAs of the default size run CTAs of SB1 sites, which spread
 // evenly: 8^3x16 Ls 8 72 -> 63 us a hop, Ls 24 218 -> 198.  With more rounds
 // the sizes are equal and the large CTAs read the links in longer runs.
+// At Ls 24 a CTA of SB1 sites is three warps, and two of them on an SM take as
+// long as the six warps of the default size (one hop: 32.9 us with one small CTA
+// an SM, 49.2 with two or one default CTA, 94.3 with three, four or two default
+// ones).  So between half a default CTA an SM and three, where the halves only add
+// overhead, the default size runs unless the launch ends in M_ee^-1, whose serial
+// sweep overlaps better in small CTAs (M_pc of 6^3x12 218 -> 194 us): H_DW of
+// 8^3x8 205 us a call, 209 in small CTAs, D_DW and D_hop equal; at 8^3x16 and
+// beyond small CTAs gain 1 to 3 % in all of them.
 constexpr long long HOP_F64_DIRS = 8192;
 constexpr long long HOP_F64_SMALL = 16 * 152;
+template <int LSV>
+inline bool hop_f64_small(const HopParams& hp, long long ctas, int sms) {
+  if (ctas >= HOP_F64_SMALL) return false;
+  return LSV != 24 || hp.inv_mode || 2 * ctas <= sms || ctas > 3 * sms;
+}
 
 // Tuning variants of the hopping kernel: (register cap, prefetch).  Variant 0
 // is the untuned default: the streaming kernel by its rule (launch_hop_stream),
@@ -1209,7 +1222,8 @@ int launch_hop_at(const HopParams& hp, int nrhs, int variant, int scalar, cudaSt
       hop_dirs_f64<LSV><<<grid, DirsCfg<LSV>::NT, 0, st>>>(hp);
       return DWF_OK;
     }
-    if ((long long)grid.x * nrhs < HOP_F64_SMALL) grid.x = (hp.Vh + HopShape<LSV>::SB1 - 1) / HopShape<LSV>::SB1;
+    if (hop_f64_small<LSV>(hp, (long long)grid.x * nrhs, hop_sms(hp)))
+      grid.x = (hp.Vh + HopShape<LSV>::SB1 - 1) / HopShape<LSV>::SB1;
   }
   if (nblocks) *nblocks = grid.x * grid.y;
   return launch_hop_ls<P, LSV>(hp, grid, variant, st);

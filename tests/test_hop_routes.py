@@ -164,6 +164,38 @@ int main() {
 """
 
 
+F64 = COMMON + r"""
+// sites per CTA of an FP64 launch of `ctas` CTAs of the default size
+template <int LS>
+int sites(int ctas, int inv, int g5) {
+  dwfk::HopParams hp;
+  std::memset(&hp, 0, sizeof(hp));
+  hp.Vh = ctas * dwfk::HopShape<LS>::SB;
+  hp.Lxh = hp.L0 = hp.L1 = 2;
+  hp.d = 3.2;
+  hp.inv_mode = inv;
+  hp.g5r5 = g5;
+  int parts = 0;
+  if (dwfk::launch_hop_at<DWF_F64, LS>(hp, 1, 0, 0, nullptr, &parts, nullptr) || parts != grid) return -1;
+  return hp.Vh / grid;
+}
+
+int main() {
+  for (int inv = 0; inv < 2; inv++)
+    for (int g5 = 0; g5 < 2; g5++) {
+      CHECK((sites<24>(76, inv, g5) == 4));                   // half a CTA an SM
+      CHECK((sites<24>(77, inv, g5) == (inv ? 4 : 8)));
+      CHECK((sites<24>(456, inv, g5) == (inv ? 4 : 8)));      // three an SM
+      CHECK((sites<24>(457, inv, g5) == 4));
+      CHECK((sites<24>(2431, inv, g5) == 4 && sites<24>(2432, inv, g5) == 8));
+      CHECK((sites<16>(100, inv, g5) == 2 && sites<8>(300, inv, g5) == 4));
+    }
+  std::printf("bad %d\n", bad);
+  return bad != 0;
+}
+"""
+
+
 def _run(tmp_path, program):
     try:
         nvcc = build.nvcc()
@@ -192,3 +224,7 @@ def test_untuned_register_cap_by_number_of_ctas(tmp_path):
     """Nothing runs under a cap that one round of CTAs does not need, and the cap
     just above a full round is not the one whose last round is empty."""
     _run(tmp_path, CAPS)
+
+
+def test_small_fp64_ctas(tmp_path):
+    _run(tmp_path, F64)
