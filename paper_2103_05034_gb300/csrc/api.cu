@@ -314,13 +314,7 @@ int launch_hop(dwf_ctx* c, const HopLaunch& h, int prec, cudaStream_t st, int* n
   hp.rhs_stride = h.rhs_stride ? h.rhs_stride : half_elems(c);
   fill_fifth(c, hp, h.mf, h.nrhs);
   if (h.reduce) {
-    const int SB = c->g.Ls >= 16 ? 8 : 128 / c->g.Ls;
-    // a partial per CTA, or per consumer warp of the streaming kernel (at most
-    // 16 on each of 152 SMs); FP64 launches of fewer than 16 * 152 CTAs run
-    // CTAs of an eighth of their sites
-    size_t nb = (size_t)((c->g.Vh + SB - 1) / SB);
-    if (nb < 8 * 16 * 152) nb = 8 * 16 * 152;
-    nb *= h.nrhs;
+    const size_t nb = dwfk::hop_partials(prec, c->g.Vh, c->g.Ls, h.nrhs, dwfk::hop_sms(hp));
     int rc = dwf_reserve_partials(c, nb);
     if (rc) return rc;
   }

@@ -1149,7 +1149,8 @@ inline bool launch_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, in
     }
     return device_sms();
   });
-  const int sms = ready ? *ready : 0;
+  int sms = ready ? *ready : 0;
+  if (hp.sms > 0 && hp.sms < sms) sms = hp.sms;  // (what the partial sums were reserved for)
   if (sms < 1 || too_small(sms)) return false;
   if (hp.inv_mode && !hp.one_sweep) return false;
   StreamGrid g;
@@ -1198,6 +1199,17 @@ bool try_hop_stream(const HopParams& hp, int nrhs, cudaStream_t st, int* nblocks
     return launch_hop_stream<P, 16, 4>(hp, nrhs, st, nblocks) || launch_hop_stream<P, 16, 3>(hp, nrhs, st, nblocks);
   if constexpr (P == DWF_F32 && LSV == 24) return launch_hop_stream<P, 24, 2>(hp, nrhs, st, nblocks);
   return false;
+}
+
+// The most partial sums that one launch leaves, all fields together: one per CTA
+// of the default size; of FP64 launches below HOP_F64_SMALL CTAs one per SB1 sites
+// (a quarter of the default at least); of FP32 arithmetic one per consumer warp of
+// the streaming kernel, 16 on each SM, and field.
+inline size_t hop_partials(int prec, long long Vh, int Ls, int nrhs, int sms) {
+  const int SB = Ls >= 16 ? 8 : 128 / Ls;
+  const size_t ctas = (size_t)((Vh + SB - 1) / SB) * nrhs;
+  const size_t other = prec == DWF_F64 ? (size_t)HOP_F64_SMALL * 4 : (size_t)16 * sms * nrhs;
+  return ctas > other ? ctas : other;
 }
 
 // A launch at Ls = LSV: variant 0 streams where its rule says so; a launch that

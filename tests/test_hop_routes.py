@@ -196,6 +196,43 @@ int main() {
 """
 
 
+PARTIALS = COMMON + r"""
+template <int P, int LS>
+void all(int prec) {
+  const int L[][4] = {{2, 2, 2, 2}, {4, 4, 4, 4}, {6, 4, 10, 6}, {8, 8, 8, 16}, {12, 12, 12, 24}, {8, 16, 16, 32}, {16, 16, 16, 32}, {24, 24, 24, 48}};
+  for (const auto& l : L)
+    for (int nrhs = 1; nrhs <= 64; nrhs += nrhs < 6 ? 1 : 29) {
+      dwfk::HopParams hp;
+      std::memset(&hp, 0, sizeof(hp));
+      hp.L0 = l[0], hp.L1 = l[1], hp.L2 = hp.zc = l[2], hp.L3 = l[3];
+      hp.Lxh = l[0] / 2;
+      hp.Vh = l[0] * l[1] * l[2] * l[3] / 2;
+      hp.d = 3.2;
+      hp.rhs_stride = (long long)hp.Vh * 12 * LS;
+      for (int inv = 0; inv < 2; inv++) {
+        hp.inv_mode = inv;
+        hp.one_sweep = 1;
+        int parts = 0;
+        dwfk::launch_hop_at<P, LS>(hp, nrhs, 0, 0, nullptr, &parts, nullptr);
+        CHECK(parts > 0 && (size_t)parts <= dwfk::hop_partials(prec, hp.Vh, LS, nrhs, 152));
+      }
+      // what a context reserves when it is made holds every small launch: no allocation on the way
+      if (nrhs <= 4 && hp.Vh * nrhs <= 65536) CHECK(dwfk::hop_partials(prec, hp.Vh, LS, nrhs, 152) <= 65536);
+    }
+}
+int main() {
+  all<DWF_F64, 8>(DWF_F64);
+  all<DWF_F64, 24>(DWF_F64);
+  all<DWF_F64, 4>(DWF_F64);
+  all<DWF_F32, 8>(DWF_F32);
+  all<DWF_F16S, 8>(DWF_F16S);
+  all<DWF_F32, 16>(DWF_F32);
+  std::printf("bad %d\n", bad);
+  return bad != 0;
+}
+"""
+
+
 def _run(tmp_path, program):
     try:
         nvcc = build.nvcc()
@@ -228,3 +265,9 @@ def test_untuned_register_cap_by_number_of_ctas(tmp_path):
 
 def test_small_fp64_ctas(tmp_path):
     _run(tmp_path, F64)
+
+
+def test_partial_sums_fit_what_is_reserved(tmp_path):
+    """The bound that a launch reserves by holds for every route, and a reduction
+    over a few fields of a small lattice needs no more than a context has."""
+    _run(tmp_path, PARTIALS)
