@@ -980,16 +980,20 @@ inline void launch_hop_v(const HopParams& hp, dim3 grid, cudaStream_t st) {
 //   many:               64, FP32 from 32 on (filter of 16^3x32 Ls 16, order 5, 3260 /
 //                       2494 / 2393 / 2328), FP16 storage, which needs half the L1
 //                       fills, from 12 on (Ls 24 8^3x144 (30) 220 / 172 / 146 / 140)
+//   a CG or Chebyshev step at the end: 64 unless its rounds are much emptier (0.85):
+//                       filter, order 5, Ls 16 8^3x64 (13.5) 960 / 781 / 794 / 761,
+//                       8^3x80 (16.8) 1155 / 965 / 915 / 977; V-cycle of 16^4 Ls 16
+//                       (27) 14.0 ms at 80, 13.5 at 64
 //   Ls 4:               96 (8x16^2x144 (30) 187 / 175 / 179 / 183)
 // Of 1076 launches and sizes timed (both types, four Ls, D_hop, M_pc, D_DW, filter
 // and CG, one and four fields, x from 1.7 to 280) this takes 0.888 of the time
 // uncapped and 0.980 of that with 64 throughout, which was up to 11 % slower than
 // uncapped between 8 and 12 CTAs an SM.
 template <int P, int LSV>
-inline int hop_default_variant(long long ctas, int sms) {
+inline int hop_default_variant(const HopParams& hp, long long ctas) {
   constexpr int T = LSV * HopShape<LSV>::SB;
   constexpr int R0 = 65536 / (T * 144), R80 = 65536 / (T * 80), R64 = 65536 / (T * 64);
-  const double x = (double)ctas / sms;
+  const double x = (double)ctas / hop_sms(hp);
   if (x <= R0) return HOP_UNCAPPED;
   if (P == DWF_F32 && x > R64 && x <= 3 * R0) {
     if (LSV == 4) return HOP_UNCAPPED;
@@ -998,7 +1002,7 @@ inline int hop_default_variant(long long ctas, int sms) {
   if (LSV == 4 && x > R64) return 1;
   if (x > (P == DWF_F32 ? 32 : 12)) return 3;
   const auto fill = [x](int r) { return x / (r * ceil(x / r)); };  // over all rounds
-  return fill(R64) > fill(R80) ? 3 : 2;
+  return fill(R64) > (hp.cheb_mode || hp.cg_mode ? 0.85 : 1.0) * fill(R80) ? 3 : 2;
 }
 
 template <int P, int LSV>
@@ -1012,7 +1016,7 @@ inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream
   } else if constexpr (P == DWF_P_DF && LSV < 16) {
     launch_hop_v<P, LSV, 0>(hp, grid, st);
   } else if constexpr (LSV < 16) {
-    switch (hop_default_variant<P, LSV>((long long)grid.x * grid.y, hop_sms(hp))) {
+    switch (hop_default_variant<P, LSV>(hp, (long long)grid.x * grid.y)) {
       case 1: launch_hop_v<P, LSV, 1>(hp, grid, st); break;
       case 2: launch_hop_v<P, LSV, 2>(hp, grid, st); break;
       case 3: launch_hop_v<P, LSV, 3>(hp, grid, st); break;
@@ -1028,7 +1032,7 @@ inline int launch_hop_ls(const HopParams& hp, dim3 grid, int variant, cudaStream
       default: launch_hop_v<P, LSV, 0>(hp, grid, st); break;
     }
   } else {
-    if (variant == 0) variant = hop_default_variant<P, LSV>((long long)grid.x * grid.y, hop_sms(hp));
+    if (variant == 0) variant = hop_default_variant<P, LSV>(hp, (long long)grid.x * grid.y);
     switch (variant) {
       case 1: launch_hop_v<P, LSV, 1>(hp, grid, st); break;
       case 2: launch_hop_v<P, LSV, 2>(hp, grid, st); break;

@@ -131,13 +131,14 @@ const void* scalar() {
 }
 // register cap that the untuned choice runs at x CTAs an SM (0: none)
 template <int P, int LS>
-int cap(double x) {
+int cap(double x, bool fused = false) {
   constexpr int SB = dwfk::HopShape<LS>::SB;
   dwfk::HopParams hp;
   std::memset(&hp, 0, sizeof(hp));
   hp.Vh = (int)(x * 152 + 0.5) * SB;
   hp.Lxh = hp.L0 = hp.L1 = 2;
-  hp.cheb_mode = 1;  // (a launch that does not stream)
+  hp.cg_mode = fused;
+  hp.inv_mode = !fused;  // (the streaming kernel leaves both to the scalar one: no single sweep)
   if (dwfk::launch_hop_at<P, LS>(hp, 1, 0, 0, nullptr, nullptr, nullptr)) return -1;
   const void* k = kernel;
   return k == scalar<P, LS, 26>() ? 0 : k == scalar<P, LS, 1>() ? 96 : k == scalar<P, LS, 2>() ? 80 : k == scalar<P, LS, 3>() ? 64 : -1;
@@ -149,6 +150,9 @@ int main() {
   const int f16_4[] = {0, 0, 80, 80, 64, 64, 96, 96, 96, 96, 96, 96, 96, 96, 96, 96, 96};
   const int f32_8[] = {0, 0, 80, 80, 64, 64, 96, 96, 80, 80, 80, 64, 80, 80, 64, 64, 64};
   const int f16_8[] = {0, 0, 80, 80, 64, 64, 80, 80, 80, 80, 80, 64, 64, 64, 64, 64, 64};
+  CHECK((cap<DWF_F32, 8>(27) == 80 && cap<DWF_F32, 8>(27, true) == 64));  // rounds 0.84 and 0.90 full
+  CHECK((cap<DWF_F32, 8>(16.8) == 80 && cap<DWF_F32, 8>(16.8, true) == 80));
+  CHECK((cap<DWF_F32, 8>(5, true) == 80 && cap<DWF_F32, 8>(7, true) == 64 && cap<DWF_F32, 8>(2, true) == 0));
   for (int i = 0; i < 17; i++) {
     const int got[4] = {cap<DWF_F32, 4>(x[i]), cap<DWF_F16S, 4>(x[i]), cap<DWF_F32, 8>(x[i]), cap<DWF_F16S, 8>(x[i])};
     const int want[4] = {f32_4[i], f16_4[i], f32_8[i], f16_8[i]};
