@@ -28,6 +28,8 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <type_traits>
+
 #include "dwf_internal.cuh"
 #include "per_device.cuh"
 
@@ -290,10 +292,14 @@ __device__ __forceinline__ void minv_row(cpx<R>* row, bool fwd, R d, R m, R kapp
 // m kappa d^-(q+1) G_last: one dependent pass and 7 operations per complex
 // number.  It is stable while |d| >= 1 and |m d^-Ls| <= 1 (the host checks);
 // elsewhere the two terms can cancel, and two opposed sweeps (12 operations)
-// are taken as in minv_row.
+// are taken as in minv_row.  In FP32 only those: the arithmetic saved is next to
+// nothing there (M_pc of 8^2x16x144 Ls 8 121 us against 125, equal at Ls 16 and 24),
+// and the second body costs every launch of the kernel (D_DW of 8^3x12 Ls 4, FP16
+// storage, 6.1 us a launch against 5.9; the pair kernel on 8^3x4 Ls 16 18.4 us an
+// M_pc against 16.5).
 template <class R, int LS>
 __device__ __forceinline__ void minv_row_inplace(cpx<R>* row, bool fwd, R d, R m, R kappa, R dls1, bool one_sweep) {
-  if (one_sweep) {
+  if (!std::is_same<R, float>::value && one_sweep) {
     const R dinv = R(1) / d;
     cpx<R> g = cmake<R>(0, 0);
 #pragma unroll 4
