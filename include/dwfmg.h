@@ -194,6 +194,12 @@ int dwf_get_hop_scalar_variant(const dwf_ctx* ctx, int prec);
 
 /* ------------------------------------------------------------------ operators */
 
+/* Reproducibility: which kernel a hopping launch runs, and so the order of its
+ * sums, depends on precision, lattice, Ls, nrhs and the tuned choice.  The same
+ * call repeated gives the same bits; a field alone and the same field among
+ * several (nrhs, or the batch of the batched solvers, which shrinks as systems
+ * converge) agree to the rounding of the precision, not in every bit. */
+
 /* Wilson hopping term, Eq. (2), between parities: out (parity out_parity) =
  * D_hop in (parity 1-out_parity), applied on every s-slice with the same
  * links.  dagger=1 applies D_hop^dag (= gamma_5 D_hop gamma_5: the spin
