@@ -1102,7 +1102,9 @@ inline bool stream_map(CUtensorMap* m, const void* base, int elem, int rank, con
 // equal near 0.63, 0.78 (Ls 24; the line stays where it was measured against
 // an earlier form, 1170 us) and 0.72.  FP16 storage halves the bytes but not the
 // arithmetic that bounds the kernel: 24^3x48 Ls 8 386 / 581, but 16^3x32 Ls 16
-// 153 / 149 and 24^3x48 Ls 24 1195 / 1147, so only Ls 8 streams.
+// 153 / 149 and 24^3x48 Ls 24 1195 / 1147, so only Ls 8 streams, and from a fill
+// of 0.80 on: 18x24x22x28 (0.68) M_pc 210 / 184, D_DW 213 / 168, 12x18x12x36 (0.80)
+// 66 / 72 and 66 / 66, 12x18x18x36 (0.84) 92 / 104 and 94 / 96.
 // The launches that end in a CG or Chebyshev step do not stream: their three
 // more fields are read by 12 to 16 warps an SM here against 32, and that costs
 // more than the hop gains: a filter of 16^3x32 Ls 16 123 us a hop if they
@@ -1110,7 +1112,7 @@ inline bool stream_map(CUtensorMap* m, const void* base, int elem, int rank, con
 // 663 us.
 template <int P, int LS>
 constexpr double stream_min_fill() {
-  return LS == 8 ? 0.68 : LS == 16 ? 0.74 : 0.87;
+  return LS == 8 ? (P == DWF_F32 ? 0.68 : 0.80) : LS == 16 ? 0.74 : 0.87;
 }
 
 // Decomposition for tiles of SX sites a row on sms CTAs; *fill as above.

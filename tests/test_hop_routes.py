@@ -237,6 +237,19 @@ int main() {
 """
 
 
+LINES = COMMON + r"""
+int main() {
+  // fills 0.68 and 0.72 (a tile's rows of six sites), 0.80, 0.84
+  CHECK((route<DWF_F32, 8>(18, 24, 22, 28, 1, 0, 0).streamed && !route<DWF_F16S, 8>(18, 24, 22, 28, 1, 0, 0).streamed));
+  CHECK((route<DWF_F32, 8>(18, 22, 24, 38, 3, 0, 0).streamed && !route<DWF_F16S, 8>(18, 22, 24, 38, 3, 0, 0).streamed));
+  CHECK((route<DWF_F32, 8>(12, 18, 12, 36, 1, 0, 0).streamed && route<DWF_F16S, 8>(12, 18, 12, 36, 1, 0, 0).streamed));
+  CHECK((route<DWF_F32, 8>(12, 18, 18, 36, 1, 0, 0).streamed && route<DWF_F16S, 8>(12, 18, 18, 36, 1, 0, 0).streamed));
+  std::printf("bad %d\n", bad);
+  return bad != 0;
+}
+"""
+
+
 def _run(tmp_path, program):
     try:
         nvcc = build.nvcc()
@@ -275,3 +288,7 @@ def test_partial_sums_fit_what_is_reserved(tmp_path):
     """The bound that a launch reserves by holds for every route, and a reduction
     over a few fields of a small lattice needs no more than a context has."""
     _run(tmp_path, PARTIALS)
+
+
+def test_streaming_line_of_fp16_storage(tmp_path):
+    _run(tmp_path, LINES)
